@@ -74,6 +74,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return mbar_wait_limit(bar, parity, abort, kWaitNs);
 }
 
+// The same for a whole warp (all 32 lanes call it): one verdict for all lanes.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return __all_sync(0xffffffffu, mbar_wait_limit(bar, parity, abort, kWaitNs));
+}
+
+// True in one lane of a converged warp, the same lane every time.  The MMA issuers run as
+// a whole warp and put only the tcgen05 instructions under this predicate: descriptors,
+// TMEM addresses and loop state then stay warp-uniform, where the instructions take them,
+// instead of being moved there from one divergent thread's registers before every MMA.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // 3-D tiled TMA load (x = innermost element index, y = row, z = head) into shared memory,
 // completing `bytes` on `bar`.
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y, int z) {

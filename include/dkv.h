@@ -40,7 +40,8 @@
  *     dkv_bank_sync() reports; CUDA launch errors are returned as
  *     DKV_ERR_CUDA by the call that saw them.
  *   - Calls on one handle must be ordered on one stream (or by the caller's
- *     own events).  admit must be followed by compress before the next admit
+ *     own events); attend calls among themselves too, since they share the
+ *     handle's attention scratch.  admit must be followed by compress before the next admit
  *     (else DKV_ERR_STATE).  attend between admit and compress reads the
  *     pre-update bank: the update is atomic from the reader's point of view
  *     (App. C, "Decision granularity versus computational tiling").
@@ -146,7 +147,9 @@ typedef struct {
   void* workspace;      /* device scratch, >= dkv_bank_workspace_size_ex() bytes for
                            the handle's parameters (= dkv_bank_workspace_size() with
                            the key descriptor), 256-byte aligned; contents are
-                           private to the handle                                    */
+                           private to the handle.  20 MB of it (bf16, d = 128, tensor
+                           mode) are attention's partial results; a workspace without
+                           them is accepted, attention then does not split units      */
   size_t workspace_bytes;
 } dkv_buffers_t;
 

@@ -112,7 +112,7 @@ void timer_end(Timer* t, cudaStream_t s) {
 // ------------------------------------------------------------------ workspace
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t ws_layout(int H, int d, int M_max, int n_max, int bf16, int kv, Ws* out, char* base) {
+size_t ws_layout(int H, int d, int M_max, int n_max, int bf16, int kv, bool attn, Ws* out, char* base) {
   const size_t es = bf16 ? 2 : 4;
   const int hist_stride = ((n_max + 2) + 3) & ~3;
   const int snap_stride = n_max / SNAP + 2;
@@ -171,6 +171,7 @@ size_t ws_layout(int H, int d, int M_max, int n_max, int bf16, int kv, Ws* out, 
   w.loop_stride = (int64_t)(Hh * std::max((Mm + 127) / 128, (Nm + 127) / 128));
   w.loop_list = (int32_t*)take(3 * (size_t)w.loop_stride * 4);
   w.loop_ctr = (int32_t*)take(3 * 2 * 4);
+  if (attn) w.attn_part = (float*)take(attend_scratch_bytes());
   w.part_stride = part_stride;
   w.cnt_stride = cnt_stride;
   w.invb_stride = invb_stride;
@@ -276,7 +277,8 @@ size_t dkv_bank_workspace_size_ex(int32_t H, int32_t d, const int32_t* budgets, 
     if (budgets[h] < 1 || budgets[h] > kMaxM) return 0;
     M_max = budgets[h] > M_max ? budgets[h] : M_max;
   }
-  return ws_layout(H, d, M_max, n_max, dtype == DKV_DTYPE_BF16, kv, nullptr, nullptr);
+  const bool attn = d == 128 && dtype == DKV_DTYPE_BF16 && (!params || params->score_mode == DKV_SCORE_TENSOR);
+  return ws_layout(H, d, M_max, n_max, dtype == DKV_DTYPE_BF16, kv, attn, nullptr, nullptr);
 }
 
 size_t dkv_bank_workspace_size(int32_t H, int32_t d, const int32_t* budgets, int32_t n_max, int32_t dtype) {
@@ -312,8 +314,11 @@ dkv_status_t dkv_bank_create(dkv_bank_t* out, int32_t H, int32_t d, const int32_
   if (!aligned(buf->k, 16) || !aligned(buf->v, 16) || !aligned(buf->workspace, 256)) return DKV_ERR_ARG;
   const int bf16 = dtype == DKV_DTYPE_BF16;
   const int kv = p.descriptor == DKV_DESC_KV;
-  const size_t need = ws_layout(H, d, M_max, n_max, bf16, kv, nullptr, nullptr);
+  // the attention scratch is optional: without room for it attention does not split units
+  const size_t need = ws_layout(H, d, M_max, n_max, bf16, kv, false, nullptr, nullptr);
   if (buf->workspace_bytes < need) return DKV_ERR_NOMEM;
+  const bool attn = p.score_mode == DKV_SCORE_TENSOR &&
+                    buf->workspace_bytes >= ws_layout(H, d, M_max, n_max, bf16, kv, true, nullptr, nullptr);
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return DKV_ERR_CUDA;
   cudaDeviceProp prop;
@@ -340,7 +345,7 @@ dkv_status_t dkv_bank_create(dkv_bank_t* out, int32_t H, int32_t d, const int32_
   b.k = buf->k; b.v = buf->v; b.rho = buf->rho; b.base = buf->base; b.knorm = buf->knorm;
   b.prov_step = buf->prov_step; b.prov_src = buf->prov_src; b.occ = buf->occupancy;
   b.H = H; b.d = d; b.M_max = M_max; b.n_max = n_max; b.bf16 = bf16;
-  ws_layout(H, d, M_max, n_max, bf16, kv, &bk->w, (char*)buf->workspace);
+  ws_layout(H, d, M_max, n_max, bf16, kv, attn, &bk->w, (char*)buf->workspace);
   bk->w.layer_heads = p.layer_heads > 0 ? p.layer_heads : H;
   bk->n_layers = H / bk->w.layer_heads;
   const float sg = bk->params.sigma;
@@ -605,7 +610,7 @@ dkv_status_t dkv_bank_attend(dkv_bank_t bank, const void* Q, int32_t Nq, const v
   if (!aligned(Q, 16) || !aligned(O, 16) || (W > 0 && (!aligned(Kw, 16) || !aligned(Vw, 16)))) return DKV_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   bank->last = s;
-  cudaError_t e = bank->tc ? launch_attend_tc(bank->b, bank->w.L, Q, Nq, Kw, Vw, W, O, s, &bank->timer)
+  cudaError_t e = bank->tc ? launch_attend_tc(bank->b, bank->w, Q, Nq, Kw, Vw, W, O, s, &bank->timer)
                            : launch_attend_fp32(bank->b, Q, Nq, Kw, Vw, W, O, s, &bank->timer);
   return cuda_status(e);
 }

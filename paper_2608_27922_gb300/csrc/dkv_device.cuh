@@ -82,6 +82,12 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 
+// Programmatic dependent launch: pdl_wait() returns once every kernel that this one was
+// launched after has completed and its writes are visible (at once in an ordinary launch);
+// pdl_trigger() allows the next kernel's blocks to start when every block has called it.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Monotone map of floats to unsigned keys (a < b  =>  fkey(a) < fkey(b); -0 below +0).
 __device__ __forceinline__ uint32_t fkey(float x) {
   uint32_t u = __float_as_uint(x);

@@ -76,6 +76,9 @@ struct Ws {
                         //   side by side), appended by the pass's classification kernel
   int32_t* loop_ctr;    // [3][2] their count, and the next one to take
   int64_t loop_stride;  // H * max(ceil(M_max / 128), ceil(n_max / 128))
+  float* attn_part;     // scratch of the tensor-core attention's split units (its own: attention
+                        //   may run beside evict), nullptr without tensor mode or in a workspace
+                        //   without room for it
   int hist_stride, snap_stride, feas_words, part_stride, cnt_stride, invb_stride, sort_stride;
   int layer_heads;      // heads per layer (the handle's heads form H / layer_heads layers)
 };
@@ -90,8 +93,9 @@ struct RopeArgs {
 // Per-layer state of head h.
 __host__ __device__ inline DevLayer* layer_of(const Ws& w, int h) { return w.L + h / w.layer_heads; }
 
-// Computes the sub-buffer offsets of the workspace; returns the total bytes.
-size_t ws_layout(int H, int d, int M_max, int n_max, int bf16, int kv, Ws* out, char* base);
+// Computes the sub-buffer offsets of the workspace; returns the total bytes.  attn: with
+// the attention scratch, the last part of the layout.
+size_t ws_layout(int H, int d, int M_max, int n_max, int bf16, int kv, bool attn, Ws* out, char* base);
 
 // Kernel timing hook (dkv_api.cu): brackets a launch with events when enabled.
 struct Timer;
@@ -136,8 +140,26 @@ cudaError_t launch_set_occupancy(const Bank& b, const int32_t* occ_dev_src, int 
 // attention
 cudaError_t launch_attend_fp32(const Bank& b, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
                                void* O, cudaStream_t s, Timer* t);
-cudaError_t launch_attend_tc(const Bank& b, DevLayer* L, const void* Q, int Nq, const void* Kw, const void* Vw,
+size_t attend_scratch_bytes();   // per handle: 20 MB of partial results
+cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw,
                              int W, void* O, cudaStream_t s, Timer* t);
+// Launches `k` so that its blocks may start before the preceding kernel of the stream has
+// ended (programmatic dependent launch): k must call pdl_wait() before it reads or writes
+// anything that kernel or an earlier one touches.
+template <typename... Args>
+cudaError_t launch_after(void (*k)(Args...), dim3 grid, unsigned threads, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 bool tc_supported(int d, int bf16);
 int sm_count();   // multiprocessors of the current device (0 if unknown)
 cudaError_t simt_set_smem_limits();

@@ -28,6 +28,8 @@
 #include "dkv_internal.h"
 #include "tc_ptx.cuh"
 
+#include <algorithm>
+#include <cmath>
 #include <climits>
 
 namespace dkv {
@@ -107,8 +109,74 @@ struct AttnJob {
   int W;
   __nv_bfloat16* O;
   float sl2;     // log2(e) / sqrt(d)
+  float* part;   // partial results of split units (nullptr: units are not split), see below
+  int4* meta;    // [CTAs] the split unit whose first part CTA i holds: {head, query tile, last
+                 //   CTA of the unit, 1}, or {.., .., .., 0}
 };
 
+// Equal shares of key tiles.  A unit is one 128-query tile of one head with all of that
+// head's key tiles (at least one: a head without keys still writes its zeros).  The key
+// tiles of all units, head-major, form one range of T tiles, and CTA i of G takes tiles
+// [i T / G, (i + 1) T / G) of it, whatever units they belong to: one unit per CTA leaves
+// most of the SMs idle in the last wave (12 heads x 1,560 queries are 156 units on 152
+// SMs), or all but a few when the units are few (one head, 128 queries: one CTA).  A unit
+// inside one CTA's share is finished there; a unit cut by a share boundary leaves fp32
+// partial results, one slot per part (part 2 i: the unit that CTA i's share begins in the
+// middle of; part 2 i + 1: the unit that it ends in the middle of), merged by tc_attend_merge.
+// A share is at least SPLIT_MIN tiles (or there is one per unit): below that a part's fixed
+// cost (query tile, first scores, partial store, about 6 us) outweighs its tiles (about 1 us
+// for two).  Units of fewer than SPLIT_UNIT tiles are not cut (a boundary inside one moves to
+// its start): they are short by themselves, and their results then do not depend on the
+// other heads of the call.
+constexpr int SPLIT_MIN = 4;
+constexpr int SPLIT_UNIT = 16;
+constexpr int SPLIT_CTAS = 152;              // most shares (the SMs of the GPU): sizes the scratch
+constexpr int PART_FLOATS = BQ * 128 + BQ;   // O [32 column groups][128 rows] float4, then lse [128]
+
+// Key tiles of a head's units.
+__device__ __forceinline__ int unit_tiles(const AttnJob& j, int h) {
+  const int m = min(max(j.b.occ[h], 0), j.b.M_max);
+  return max(1, (m + BK - 1) / BK + (j.W + BK - 1) / BK);
+}
+
+// One CTA's position in the range: the head `h` whose tiles begin at `base`.  All lanes of
+// one warp call seek together; 32 heads are looked at at a time.
+struct TileCursor {
+  int h, base;
+  __device__ __forceinline__ int seek(const AttnJob& j, int nqt, int t) {   // -> tiles per unit of head h
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+      const int hh = h + lane;
+      const int n = hh < j.b.H ? unit_tiles(j, hh) : 0;
+      int incl = n * nqt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const unsigned past = __ballot_sync(0xffffffffu, hh < j.b.H && base + incl > t);
+      if (past) {
+        const int k = __ffs(past) - 1;
+        const int before = __shfl_sync(0xffffffffu, incl - n * nqt, k);
+        const int nt = __shfl_sync(0xffffffffu, n, k);
+        h += k;
+        base += before;
+        return nt;
+      }
+      base += __shfl_sync(0xffffffffu, incl, 31);
+      h += 32;
+      if (h >= j.b.H) return 0;   // past the end
+    }
+  }
+  // Share boundary t, 0 <= t <= total, moved to the start of its unit if that is not cut.
+  __device__ __forceinline__ int snap(const AttnJob& j, int nqt, int t, int total) {
+    if (t >= total) return total;
+    const int su = seek(j, nqt, t);
+    return su < SPLIT_UNIT ? t - (t - base) % su : t;
+  }
+};
+
+template <bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_attend(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKb,
               const __grid_constant__ CUtensorMap tmVb, const __grid_constant__ CUtensorMap tmKw,
@@ -130,17 +198,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* pv_done = bars + 13;  // [2]
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 15);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  volatile int* seg = reinterpret_cast<volatile int*>(tmem_holder + 2);   // [5] the segment, see below
 
-  const int h = blockIdx.y;
-  const int q0 = blockIdx.x * BQ;
-  const int m = min(max(j.b.occ[h], 0), j.b.M_max);
-  const int W = j.W;
-  const int nb = (m + BK - 1) / BK;            // bank tiles
-  const int nt = nb + (W + BK - 1) / BK;       // all key tiles
-  const int nh = (nt + 1) / 2;                 // tiles of group 0; group 1 takes the rest
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-  if (threadIdx.x == 0) {
+  const int W = j.W;
+  const int nqt = (j.Nq + BQ - 1) / BQ;
+  auto init_bars = [&]() {
     mbar_init(q_full, 1);
     for (int g = 0; g < 2; ++g) {
       mbar_init(k0_full + g, 1);
@@ -150,285 +213,437 @@ __global__ void __launch_bounds__(THREADS, 1)
       mbar_init(p_full + g, 4 + 1);   // four softmax warps + the producer (with bytes)
       mbar_init(pv_done + g, 1);
     }
-    *abort_flag = 0;
     fence_barrier_init();
-  }
+  };
   if (warp == 1) tmem_alloc(tmem_holder, TMEM_COLS);
+  // SPLIT: this CTA's share of the range (warp 0 only)
+  int lo = 0, hi = 0, total = 0, shares = 1;
+  TileCursor cur{0, 0};
+  if (SPLIT) {
+    pdl_trigger();   // the merge's blocks start as SMs free up, and wait there
+    if (warp == 0) {
+      int mine = 0;
+      for (int hh = lane; hh < j.b.H; hh += 32) mine += unit_tiles(j, hh);
+      total = __reduce_add_sync(0xffffffffu, mine) * nqt;
+      shares = min((int)gridDim.x, max(j.b.H * nqt, total / SPLIT_MIN));
+      if ((int)blockIdx.x < shares) {
+        lo = cur.snap(j, nqt, (int)((int64_t)blockIdx.x * total / shares), total);
+        TileCursor end = cur;
+        hi = end.snap(j, nqt, (int)((int64_t)(blockIdx.x + 1) * total / shares), total);
+      }
+      if (lane == 0) j.meta[blockIdx.x] = make_int4(0, 0, 0, 0);
+    }
+  }
+  if (threadIdx.x == 0) {
+    *abort_flag = 0;
+    if (!SPLIT) init_bars();
+  }
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = *tmem_holder;
 
-  auto tiles_of = [&](int g) { return g == 0 ? nh : nt - nh; };
-  auto tile_index = [&](int g, int i) { return g * nh + i; };
+  for (;;) {
+    // ---- the segment: tiles [first, first + nseg) of the unit of head h, query tile qt, which
+    // has nt_unit tiles in all; one whole unit without SPLIT
+    int h, qt, first = 0, nseg, nt_unit;
+    if (SPLIT) {
+      if (warp == 0) {
+        int sh = -1, sq = 0, sa = 0, sn = 0, su = 0;
+        if (lo < hi) {
+          su = cur.seek(j, nqt, lo);
+          sh = cur.h;
+          sq = (lo - cur.base) / su;
+          sa = (lo - cur.base) - sq * su;
+          sn = min(su - sa, hi - lo);
+          if (lane == 0 && sa == 0 && sn < su) {   // first part of a cut unit: its last CTA
+            const int64_t end = (int64_t)(lo + su) * shares;
+            j.meta[blockIdx.x] = make_int4(sh, sq, (int)((end + total - 1) / total) - 1, 1);
+          }
+          lo += sn;
+        }
+        if (lane == 0) {
+          seg[0] = sh; seg[1] = sq; seg[2] = sa; seg[3] = sn; seg[4] = su;
+          init_bars();
+        }
+      }
+      __syncthreads();
+      h = seg[0];
+      if (h < 0) break;                          // uniform
+      qt = seg[1]; first = seg[2]; nseg = seg[3]; nt_unit = seg[4];
+    } else {
+      h = blockIdx.x / nqt;
+      qt = blockIdx.x - h * nqt;
+      nseg = nt_unit = unit_tiles(j, h);
+    }
+    const int q0 = qt * BQ;
+    const int m = min(max(j.b.occ[h], 0), j.b.M_max);
+    const int nb = (m + BK - 1) / BK;            // bank tiles of the unit
+    // a head without keys has one tile in the range and none to load
+    const int nt = nb + W > 0 ? nseg : 0;
+    const int nh = (nt + 1) / 2;                 // tiles of group 0; group 1 takes the rest
 
-  if (warp == 0) {
-    if (lane == 0 && nt > 0) {
-      // ---------------- TMA producer: Q once; per group K(0), then for each tile i the
-      // bytes of V(i) and K(i + 1) on p_full_g (phase i)
-      prefetch_map(&tmQ);
-      mbar_arrive_expect_tx(q_full, TB);
-      tma_load_3d(smem + OFF_Q, &tmQ, q_full, 0, q0, h);
-      tma_load_3d(smem + OFF_Q + HB, &tmQ, q_full, 64, q0, h);
-      const int n[2] = {tiles_of(0), tiles_of(1)};
-      auto load_tile = [&](bool is_k, int g, int i, void* dst, uint64_t* bar) {
+    auto tiles_of = [&](int g) { return g == 0 ? nh : nt - nh; };
+    auto tile_index = [&](int g, int i) { return first + g * nh + i; };
+
+    if (warp == 0) {
+      if (lane == 0 && nt > 0) {
+        // ---------------- TMA producer: Q once; per group K(0), then for each tile i the
+        // bytes of V(i) and K(i + 1) on p_full_g (phase i)
+        prefetch_map(&tmQ);
+        mbar_arrive_expect_tx(q_full, TB);
+        tma_load_3d(smem + OFF_Q, &tmQ, q_full, 0, q0, h);
+        tma_load_3d(smem + OFF_Q + HB, &tmQ, q_full, 64, q0, h);
+        const int n[2] = {tiles_of(0), tiles_of(1)};
+        auto load_tile = [&](bool is_k, int g, int i, void* dst, uint64_t* bar) {
+          const int u = tile_index(g, i);
+          const bool bank = u < nb;
+          const CUtensorMap* mp = is_k ? (bank ? &tmKb : &tmKw) : (bank ? &tmVb : &tmVw);
+          const int row = bank ? u * BK : (u - nb) * BK;
+          tma_load_3d(dst, mp, bar, 0, row, h);
+          tma_load_3d(static_cast<uint8_t*>(dst) + HB, mp, bar, 64, row, h);
+        };
+        for (int g = 0; g < 2; ++g)
+          if (n[g] > 0) {
+            mbar_arrive_expect_tx(k0_full + g, TB);
+            load_tile(true, g, 0, smem + OFF_K + (2 * g) * TB, k0_full + g);
+          }
+        int armed[2] = {0, 0};   // p_full phases armed per group
+        bool ok = true;
+        for (int i = 0; ok && i < n[0]; ++i) {
+          for (int g = 0; g < 2 && ok; ++g) {
+            if (i >= n[g]) continue;
+            // PV_g(i - 1) complete: the V slot is free and p_full_g phase i - 1 is over
+            if (i > 0 && !(ok = mbar_wait(v_empty + g, (i - 1) & 1, abort_flag))) break;
+            const bool knext = i + 1 < n[g];
+            // S_g(i - 1) complete: K slot (i + 1) & 1 is free
+            if (knext && i > 0 && !(ok = mbar_wait(k_empty + 2 * g + ((i + 1) & 1), ((i - 1) >> 1) & 1, abort_flag)))
+              break;
+            mbar_arrive_expect_tx(p_full + g, knext ? 2 * TB : TB);
+            load_tile(false, g, i, smem + OFF_V + g * TB, p_full + g);
+            if (knext) load_tile(true, g, i + 1, smem + OFF_K + (2 * g + ((i + 1) & 1)) * TB, p_full + g);
+            armed[g] = i + 1;
+          }
+        }
+        if (!ok) {
+          *abort_flag = 1;
+          dev_fail(j.L, DEV_TIMEOUT, 400);
+        }
+        // never leave with copies in flight: earlier phases completed before this thread
+        // armed the next one; the last armed phase also needs the softmax, which an
+        // aborted CTA may never give: then wait a fixed 50 us, far longer than a copy takes
+        volatile int no_abort = 0;
+        mbar_wait(q_full, 0, &no_abort);
+        bool drained = true;
+        for (int g = 0; g < 2; ++g) {
+          if (n[g] > 0) mbar_wait(k0_full + g, 0, &no_abort);
+          if (armed[g] > 0) drained = drained && mbar_wait(p_full + g, (armed[g] - 1) & 1, abort_flag);
+        }
+        if (!drained) {
+          const uint64_t t0 = globaltimer_ns();
+          while (globaltimer_ns() - t0 < 50000ull) {
+          }
+        }
+      }
+    } else if (warp == 1) {
+      if (nt > 0) {
+        // ---------------- MMA issuer (the whole warp, one elected lane issues).  Per group:
+        // S(0), then for each tile i:
+        // PV(i) once P(i) is in TMEM, then S(i+1) (which overwrites P(i) after PV(i) read it).
+        constexpr uint32_t id_s = idesc_bf16(BQ, BK);
+        constexpr uint32_t id_o = idesc_bf16(BQ, 128, /*b_mn_major=*/true);
+        const uint32_t q_base = smem_u32(smem + OFF_Q);
+        const int n[2] = {tiles_of(0), tiles_of(1)};
+        bool ok = mbar_wait_warp(q_full, 0, abort_flag);
+        int pv_issued[2] = {0, 0};
+        // S_g(i): its K tile has landed (K(0): k0_full; K(i + 1): with p_full_g phase i)
+        const uint64_t qd = desc_sw128(q_base), kd0 = desc_sw128(smem_u32(smem + OFF_K));
+        const uint64_t vd0 = desc_sw128_mn(smem_u32(smem + OFF_V), HB, 1024);
+        auto issue_s = [&](int g, int i) {
+          const uint64_t kd = desc_add(kd0, (2 * g + (i & 1)) * TB);
+          const uint32_t sc = tmem + g * 256;
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+              const uint32_t off = (kk >> 2) * HB + (kk & 3) * 32;
+              mma_bf16(sc, desc_add(qd, off), desc_add(kd, off), id_s, kk > 0);
+            }
+            mma_commit(k_empty + 2 * g + (i & 1));
+            mma_commit(s_full + g);
+          }
+          __syncwarp();
+        };
+        auto issue_pv = [&](int g, int i) -> bool {
+          if (!mbar_wait_warp(p_full + g, i & 1, abort_flag)) return false;   // the one wait
+          fence_after_sync();
+          const uint64_t vd = desc_add(vd0, g * TB);
+          const uint32_t pc = tmem + g * 256;          // P: packed bf16 pairs over S columns [0, 64)
+          const uint32_t oc = tmem + g * 256 + 128;
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk)
+              mma_bf16_ts(oc, pc + kk * 8, desc_add(vd, kk * 2048), id_o, (i > 0 || kk > 0) ? 1u : 0u);
+            mma_commit(v_empty + g);
+            mma_commit(pv_done + g);
+          }
+          __syncwarp();
+          pv_issued[g] = i + 1;
+          return true;
+        };
+        for (int g = 0; g < 2 && ok; ++g)
+          if (n[g] > 0) {
+            if ((ok = mbar_wait_warp(k0_full + g, 0, abort_flag))) {
+              fence_after_sync();
+              issue_s(g, 0);
+            }
+          }
+        for (int i = 0; ok && i < n[0]; ++i) {
+          for (int g = 0; g < 2 && ok; ++g) {
+            if (i >= n[g]) continue;
+            ok = issue_pv(g, i);
+            if (ok && i + 1 < n[g]) issue_s(g, i + 1);
+          }
+        }
+        if (!ok && lane == 0) {
+          *abort_flag = 1;
+          dev_fail(j.L, DEV_TIMEOUT, 401);
+        }
+        volatile int no_abort = 0;
+        for (int g = 0; g < 2; ++g)
+          if (pv_issued[g] > 0) mbar_wait(pv_done + g, (pv_issued[g] - 1) & 1, &no_abort);
+      }
+    } else {
+      // ---------------- softmax group g, thread = query row = TMEM lane
+      const int g = (warp - 2) >> 2;
+      const int qd = warp & 3;
+      const int r = qd * 32 + lane;
+      const uint32_t lane_off = (uint32_t)(qd * 32) << 16;
+      const uint32_t sc = tmem + lane_off + g * 256;     // S_g (and P_g)
+      const uint32_t oc = sc + 128;                      // O_g
+      const int ng = tiles_of(g);
+      float mrun = -INFINITY, l = 0.f;
+      bool ok = true;
+      for (int i = 0; i < ng; ++i) {
         const int u = tile_index(g, i);
         const bool bank = u < nb;
-        const CUtensorMap* mp = is_k ? (bank ? &tmKb : &tmKw) : (bank ? &tmVb : &tmVw);
-        const int row = bank ? u * BK : (u - nb) * BK;
-        tma_load_3d(dst, mp, bar, 0, row, h);
-        tma_load_3d(static_cast<uint8_t*>(dst) + HB, mp, bar, 64, row, h);
-      };
-      for (int g = 0; g < 2; ++g)
-        if (n[g] > 0) {
-          mbar_arrive_expect_tx(k0_full + g, TB);
-          load_tile(true, g, 0, smem + OFF_K + (2 * g) * TB, k0_full + g);
+        const int valid = bank ? min(BK, m - u * BK) : min(BK, W - (u - nb) * BK);
+        ok = ok && __all_sync(0xffffffffu, mbar_wait(s_full + g, i & 1, abort_flag));
+        if (!ok) break;
+        fence_after_sync();
+        // the whole row of S_g (128 scores) in registers: four loads, one wait
+        float s0[32], s1[32], s2[32], s3[32];
+        tmem_ld32(sc, s0);
+        tmem_ld32(sc + 32, s1);
+        tmem_ld32(sc + 64, s2);
+        tmem_ld32(sc + 96, s3);
+        tmem_wait_ld();
+        if (valid < BK) {   // partial last tile of the bank or of the window
+          mask_tail(s0, valid); mask_tail(s1, valid - 32); mask_tail(s2, valid - 64); mask_tail(s3, valid - 96);
         }
-      int armed[2] = {0, 0};   // p_full phases armed per group
-      bool ok = true;
-      for (int i = 0; ok && i < n[0]; ++i) {
-        for (int g = 0; g < 2 && ok; ++g) {
-          if (i >= n[g]) continue;
-          // PV_g(i - 1) complete: the V slot is free and p_full_g phase i - 1 is over
-          if (i > 0 && !(ok = mbar_wait(v_empty + g, (i - 1) & 1, abort_flag))) break;
-          const bool knext = i + 1 < n[g];
-          // S_g(i - 1) complete: K slot (i + 1) & 1 is free
-          if (knext && i > 0 && !(ok = mbar_wait(k_empty + 2 * g + ((i + 1) & 1), ((i - 1) >> 1) & 1, abort_flag)))
-            break;
-          mbar_arrive_expect_tx(p_full + g, knext ? 2 * TB : TB);
-          load_tile(false, g, i, smem + OFF_V + g * TB, p_full + g);
-          if (knext) load_tile(true, g, i + 1, smem + OFF_K + (2 * g + ((i + 1) & 1)) * TB, p_full + g);
-          armed[g] = i + 1;
+        // row maximum of the raw scores
+        float tmax;
+        {
+          float t[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) t[k] = -INFINITY;
+          max_acc(t, s0); max_acc(t, s1); max_acc(t, s2); max_acc(t, s3);
+          tmax = fmaxf(fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3])), fmaxf(fmaxf(t[4], t[5]), fmaxf(t[6], t[7])));
         }
+        tmax *= j.sl2;
+        // lazily raised running maximum.  S_g(i) complete implies PV_g(i-1) complete
+        // (one thread issues both, in order), so O_g is idle here.
+        const bool raise = tmax > mrun + RESCALE_LOG2;
+        const float mnew = raise ? tmax : mrun;
+        const float mprev = mrun;
+        if (raise) {
+          l *= (i > 0) ? ex2(mrun - mnew) : 0.f;
+          mrun = mnew;
+        }
+        // P_g = 2^(s log2(e)/sqrt(d) - m) as packed bf16 pairs over the first 64 columns of S_g
+        const float nm = -mrun;
+        float2 lab = make_float2(0.f, 0.f);     // running sums of the even and odd columns
+        {
+          uint32_t pk[32];
+          exp_pack(s0, s1, j.sl2, nm, lab, pk);
+          tmem_st32(sc, pk);
+          exp_pack(s2, s3, j.sl2, nm, lab, pk);
+          tmem_st32(sc + 32, pk);
+        }
+        // O_g rescale: after the P stores (S is dead), before PV(i) is released
+        if (__any_sync(0xffffffffu, raise && i > 0)) {
+          const float alpha = raise ? ex2(mprev - mnew) : 1.0f;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            float v[32];
+            tmem_ld32(oc + c * 32, v);
+            tmem_wait_ld();
+            uint32_t w32[32];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+              const float2 y = __fmul2_rn(make_float2(v[2 * k], v[2 * k + 1]), make_float2(alpha, alpha));
+              w32[2 * k] = __float_as_uint(y.x);
+              w32[2 * k + 1] = __float_as_uint(y.y);
+            }
+            tmem_st32(oc + c * 32, w32);
+          }
+        }
+        l += lab.x + lab.y;
+        tmem_wait_st();
+        fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full + g);
       }
+      // ---- merge the two groups' partial softmax results
+      if (ok && ng > 0) ok = __all_sync(0xffffffffu, mbar_wait(pv_done + g, (ng - 1) & 1, abort_flag));
       if (!ok) {
         *abort_flag = 1;
-        dev_fail(j.L, DEV_TIMEOUT, 400);
+        if (lane == 0) dev_fail(j.L, DEV_TIMEOUT, 402);
       }
-      // never leave with copies in flight: earlier phases completed before this thread
-      // armed the next one; the last armed phase also needs the softmax, which an
-      // aborted CTA may never give: then wait a fixed 50 us, far longer than a copy takes
-      volatile int no_abort = 0;
-      mbar_wait(q_full, 0, &no_abort);
-      bool drained = true;
-      for (int g = 0; g < 2; ++g) {
-        if (n[g] > 0) mbar_wait(k0_full + g, 0, &no_abort);
-        if (armed[g] > 0) drained = drained && mbar_wait(p_full + g, (armed[g] - 1) & 1, abort_flag);
+      xst[(g * 2 + 0) * BQ + r] = ng > 0 && ok ? mrun : -INFINITY;
+      xst[(g * 2 + 1) * BQ + r] = ng > 0 && ok ? l : 0.f;
+      named_bar(1 + qd, 64);   // the two warps (one per group) of this TMEM lane quarter
+      const float m0 = xst[0 * BQ + r], l0 = xst[1 * BQ + r];
+      const float m1 = xst[2 * BQ + r], l1 = xst[3 * BQ + r];
+      const float mm = fmaxf(m0, m1);
+      const float a0 = m0 == -INFINITY ? 0.f : ex2(m0 - mm);
+      const float a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
+      const float den = fmaf(a1, l1, a0 * l0);
+      const float inv = den > 0.f ? 1.0f / den : 0.f;
+      const float c0 = a0 * inv, c1 = a1 * inv;
+      // the merge reads the other group's O too: observe its last PV completion as well
+      {
+        const int no = tiles_of(g ^ 1);
+        if (ok && no > 0) ok = __all_sync(0xffffffffu, mbar_wait(pv_done + (g ^ 1), (no - 1) & 1, abort_flag));
       }
-      if (!drained) {
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 50000ull) {
-        }
-      }
-    }
-  } else if (warp == 1) {
-    if (nt > 0) {
-      // ---------------- MMA issuer (the whole warp, one elected lane issues).  Per group: S(0), then for each tile i:
-      // PV(i) once P(i) is in TMEM, then S(i+1) (which overwrites P(i) after PV(i) read it).
-      constexpr uint32_t id_s = idesc_bf16(BQ, BK);
-      constexpr uint32_t id_o = idesc_bf16(BQ, 128, /*b_mn_major=*/true);
-      const uint32_t q_base = smem_u32(smem + OFF_Q);
-      const int n[2] = {tiles_of(0), tiles_of(1)};
-      bool ok = mbar_wait_warp(q_full, 0, abort_flag);
-      int pv_issued[2] = {0, 0};
-      // S_g(i): its K tile has landed (K(0): k0_full; K(i + 1): with p_full_g phase i)
-      const uint64_t qd = desc_sw128(q_base), kd0 = desc_sw128(smem_u32(smem + OFF_K));
-      const uint64_t vd0 = desc_sw128_mn(smem_u32(smem + OFF_V), HB, 1024);
-      auto issue_s = [&](int g, int i) {
-        const uint64_t kd = desc_add(kd0, (2 * g + (i & 1)) * TB);
-        const uint32_t sc = tmem + g * 256;
-        if (elect_one()) {
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint32_t off = (kk >> 2) * HB + (kk & 3) * 32;
-            mma_bf16(sc, desc_add(qd, off), desc_add(kd, off), id_s, kk > 0);
-          }
-          mma_commit(k_empty + 2 * g + (i & 1));
-          mma_commit(s_full + g);
-        }
-        __syncwarp();
-      };
-      auto issue_pv = [&](int g, int i) -> bool {
-        if (!mbar_wait_warp(p_full + g, i & 1, abort_flag)) return false;   // the one wait
-        fence_after_sync();
-        const uint64_t vd = desc_add(vd0, g * TB);
-        const uint32_t pc = tmem + g * 256;          // P: packed bf16 pairs over S columns [0, 64)
-        const uint32_t oc = tmem + g * 256 + 128;
-        if (elect_one()) {
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk)
-            mma_bf16_ts(oc, pc + kk * 8, desc_add(vd, kk * 2048), id_o, (i > 0 || kk > 0) ? 1u : 0u);
-          mma_commit(v_empty + g);
-          mma_commit(pv_done + g);
-        }
-        __syncwarp();
-        pv_issued[g] = i + 1;
-        return true;
-      };
-      for (int g = 0; g < 2 && ok; ++g)
-        if (n[g] > 0) {
-          if ((ok = mbar_wait_warp(k0_full + g, 0, abort_flag))) {
-            fence_after_sync();
-            issue_s(g, 0);
-          }
-        }
-      for (int i = 0; ok && i < n[0]; ++i) {
-        for (int g = 0; g < 2 && ok; ++g) {
-          if (i >= n[g]) continue;
-          ok = issue_pv(g, i);
-          if (ok && i + 1 < n[g]) issue_s(g, i + 1);
-        }
-      }
-      if (!ok && lane == 0) {
-        *abort_flag = 1;
-        dev_fail(j.L, DEV_TIMEOUT, 401);
-      }
-      volatile int no_abort = 0;
-      for (int g = 0; g < 2; ++g)
-        if (pv_issued[g] > 0) mbar_wait(pv_done + g, (pv_issued[g] - 1) & 1, &no_abort);
-    }
-  } else {
-    // ---------------- softmax group g, thread = query row = TMEM lane
-    const int g = (warp - 2) >> 2;
-    const int qd = warp & 3;
-    const int r = qd * 32 + lane;
-    const uint32_t lane_off = (uint32_t)(qd * 32) << 16;
-    const uint32_t sc = tmem + lane_off + g * 256;     // S_g (and P_g)
-    const uint32_t oc = sc + 128;                      // O_g
-    const int ng = tiles_of(g);
-    float mrun = -INFINITY, l = 0.f;
-    bool ok = true;
-    for (int i = 0; i < ng; ++i) {
-      const int u = tile_index(g, i);
-      const bool bank = u < nb;
-      const int valid = bank ? min(BK, m - u * BK) : min(BK, W - (u - nb) * BK);
-      ok = ok && __all_sync(0xffffffffu, mbar_wait(s_full + g, i & 1, abort_flag));
-      if (!ok) break;
       fence_after_sync();
-      // the whole row of S_g (128 scores) in registers: four loads, one wait
-      float s0[32], s1[32], s2[32], s3[32];
-      tmem_ld32(sc, s0);
-      tmem_ld32(sc + 32, s1);
-      tmem_ld32(sc + 64, s2);
-      tmem_ld32(sc + 96, s3);
-      tmem_wait_ld();
-      if (valid < BK) {   // partial last tile of the bank or of the window
-        mask_tail(s0, valid); mask_tail(s1, valid - 32); mask_tail(s2, valid - 64); mask_tail(s3, valid - 96);
-      }
-      // row maximum of the raw scores
-      float tmax;
-      {
-        float t[8];
+      // group g writes output columns [64 g, 64 g + 64) of this row from both O_0 and O_1
+      const int qrow = q0 + r;
+      const uint32_t o0 = tmem + lane_off + 128 + g * 64;
+      const uint32_t o1 = tmem + lane_off + 256 + 128 + g * 64;
+      const bool has0 = ok && tiles_of(0) > 0 && c0 != 0.f, has1 = ok && tiles_of(1) > 0 && c1 != 0.f;
+      const bool whole = !SPLIT || nseg == nt_unit;   // CTA-uniform
+      // a part of a split unit: normalised O in fp32 and the base-2 logarithm of its weight
+      float* part = whole ? nullptr : j.part + (int64_t)(2 * blockIdx.x + (first == 0 ? 1 : 0)) * PART_FLOATS;
+      if (!whole && g == 0) part[BQ * 128 + r] = den == 0.f ? -INFINITY : mm + log2f(den);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) t[k] = -INFINITY;
-        max_acc(t, s0); max_acc(t, s1); max_acc(t, s2); max_acc(t, s3);
-        tmax = fmaxf(fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3])), fmaxf(fmaxf(t[4], t[5]), fmaxf(t[6], t[7])));
-      }
-      tmax *= j.sl2;
-      // lazily raised running maximum.  S_g(i) complete implies PV_g(i-1) complete
-      // (one thread issues both, in order), so O_g is idle here.
-      const bool raise = tmax > mrun + RESCALE_LOG2;
-      const float mnew = raise ? tmax : mrun;
-      const float mprev = mrun;
-      if (raise) {
-        l *= (i > 0) ? ex2(mrun - mnew) : 0.f;
-        mrun = mnew;
-      }
-      // P_g = 2^(s log2(e)/sqrt(d) - m) as packed bf16 pairs over the first 64 columns of S_g
-      const float nm = -mrun;
-      float2 lab = make_float2(0.f, 0.f);     // running sums of the even and odd columns
-      {
-        uint32_t pk[32];
-        exp_pack(s0, s1, j.sl2, nm, lab, pk);
-        tmem_st32(sc, pk);
-        exp_pack(s2, s3, j.sl2, nm, lab, pk);
-        tmem_st32(sc + 32, pk);
-      }
-      // O_g rescale: after the P stores (S is dead), before PV(i) is released
-      if (__any_sync(0xffffffffu, raise && i > 0)) {
-        const float alpha = raise ? ex2(mprev - mnew) : 1.0f;
+      for (int c = 0; c < 2; ++c) {
+        float x0[32], x1[32];
+        tmem_ld32(o0 + c * 32, x0);
+        tmem_ld32(o1 + c * 32, x1);
+        tmem_wait_ld();
+        if (!whole) {
+          float4* dst = reinterpret_cast<float4*>(part) + (g * 16 + c * 8) * BQ + r;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          float v[32];
-          tmem_ld32(oc + c * 32, v);
-          tmem_wait_ld();
-          uint32_t w32[32];
+          for (int k = 0; k < 8; ++k) {
+            float y[4];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const float2 y = __fmul2_rn(make_float2(v[2 * k], v[2 * k + 1]), make_float2(alpha, alpha));
-            w32[2 * k] = __float_as_uint(y.x);
-            w32[2 * k + 1] = __float_as_uint(y.y);
+            for (int e = 0; e < 4; ++e) {
+              const float t0 = has0 ? x0[k * 4 + e] * c0 : 0.f;
+              y[e] = has1 ? fmaf(x1[k * 4 + e], c1, t0) : t0;
+            }
+            dst[k * BQ] = make_float4(y[0], y[1], y[2], y[3]);
           }
-          tmem_st32(oc + c * 32, w32);
-        }
-      }
-      l += lab.x + lab.y;
-      tmem_wait_st();
-      fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(p_full + g);
-    }
-    // ---- merge the two groups' partial softmax results
-    if (ok && ng > 0) ok = __all_sync(0xffffffffu, mbar_wait(pv_done + g, (ng - 1) & 1, abort_flag));
-    if (!ok) {
-      *abort_flag = 1;
-      if (lane == 0) dev_fail(j.L, DEV_TIMEOUT, 402);
-    }
-    xst[(g * 2 + 0) * BQ + r] = ng > 0 && ok ? mrun : -INFINITY;
-    xst[(g * 2 + 1) * BQ + r] = ng > 0 && ok ? l : 0.f;
-    named_bar(1 + qd, 64);   // the two warps (one per group) of this TMEM lane quarter
-    const float m0 = xst[0 * BQ + r], l0 = xst[1 * BQ + r];
-    const float m1 = xst[2 * BQ + r], l1 = xst[3 * BQ + r];
-    const float mm = fmaxf(m0, m1);
-    const float a0 = m0 == -INFINITY ? 0.f : ex2(m0 - mm);
-    const float a1 = m1 == -INFINITY ? 0.f : ex2(m1 - mm);
-    const float den = fmaf(a1, l1, a0 * l0);
-    const float inv = den > 0.f ? 1.0f / den : 0.f;
-    const float c0 = a0 * inv, c1 = a1 * inv;
-    // the merge reads the other group's O too: observe its last PV completion as well
-    {
-      const int no = tiles_of(g ^ 1);
-      if (ok && no > 0) ok = __all_sync(0xffffffffu, mbar_wait(pv_done + (g ^ 1), (no - 1) & 1, abort_flag));
-    }
-    fence_after_sync();
-    // group g writes output columns [64 g, 64 g + 64) of this row from both O_0 and O_1
-    const int qrow = q0 + r;
-    const uint32_t o0 = tmem + lane_off + 128 + g * 64;
-    const uint32_t o1 = tmem + lane_off + 256 + 128 + g * 64;
-    const bool has0 = ok && tiles_of(0) > 0 && c0 != 0.f, has1 = ok && tiles_of(1) > 0 && c1 != 0.f;
+        } else if (qrow < j.Nq) {
+          uint4* dst = reinterpret_cast<uint4*>(j.O + ((int64_t)h * j.Nq + qrow) * 128 + g * 64 + c * 32);
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      float x0[32], x1[32];
-      tmem_ld32(o0 + c * 32, x0);
-      tmem_ld32(o1 + c * 32, x1);
-      tmem_wait_ld();
-      if (qrow < j.Nq) {
-        uint4* dst = reinterpret_cast<uint4*>(j.O + ((int64_t)h * j.Nq + qrow) * 128 + g * 64 + c * 32);
+          for (int k = 0; k < 4; ++k) {
+            float y[8];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          float y[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float t0 = has0 ? x0[k * 8 + e] * c0 : 0.f;
-            y[e] = has1 ? fmaf(x1[k * 8 + e], c1, t0) : t0;
+            for (int e = 0; e < 8; ++e) {
+              const float t0 = has0 ? x0[k * 8 + e] * c0 : 0.f;
+              y[e] = has1 ? fmaf(x1[k * 8 + e], c1, t0) : t0;
+            }
+            uint4 pk;
+            pk.x = pack_bf16(y[0], y[1]);
+            pk.y = pack_bf16(y[2], y[3]);
+            pk.z = pack_bf16(y[4], y[5]);
+            pk.w = pack_bf16(y[6], y[7]);
+            dst[k] = pk;
           }
-          uint4 pk;
-          pk.x = pack_bf16(y[0], y[1]);
-          pk.y = pack_bf16(y[2], y[3]);
-          pk.z = pack_bf16(y[4], y[5]);
-          pk.w = pack_bf16(y[6], y[7]);
-          dst[k] = pk;
         }
       }
     }
+    // ---- segment end: nothing is in flight; the barriers may be initialised again
+    fence_before_sync();
+    __syncthreads();
+    if (!SPLIT) break;
+    const bool stop = *abort_flag != 0;
+    if (threadIdx.x == 0) {
+      mbar_inval(q_full);
+      for (int g = 0; g < 2; ++g) {
+        mbar_inval(k0_full + g);
+        mbar_inval(k_empty + 2 * g); mbar_inval(k_empty + 2 * g + 1);
+        mbar_inval(v_empty + g);
+        mbar_inval(s_full + g);
+        mbar_inval(p_full + g);
+        mbar_inval(pv_done + g);
+      }
+    }
+    __syncthreads();
+    if (stop) break;   // uniform
   }
-  fence_before_sync();
-  __syncthreads();
   if (warp == 1) {
     fence_after_sync();
     tmem_dealloc(tmem, TMEM_COLS);
   }
 }
+
+// O of the units that share boundaries cut: CTA (i, y) takes rows [8 y, 8 y + 8) of the unit
+// whose first part CTA i of tc_attend holds (its last segment), the parts i, i + 1, .., last
+// added in that order with weights 2^(lse - max lse).  Thread = (row, four columns).  A row
+// whose weight is not finite in some part is 0, as a row whose sum is not is in one piece.
+constexpr int MG_ROWS = 8;
+constexpr int MG_UNROLL = 4;
+
+__global__ void __launch_bounds__(MG_ROWS * 32) tc_attend_merge(AttnJob j) {
+  pdl_wait();
+  const int i = blockIdx.x;
+  const int4 u = j.meta[i];
+  if (u.w == 0) return;
+  const int n = u.z - i + 1;                   // parts
+  const int row = blockIdx.y * MG_ROWS + threadIdx.x % MG_ROWS, c4 = threadIdx.x / MG_ROWS;
+  const int qrow = u.y * BQ + row;
+  if (qrow >= j.Nq) return;
+  auto slot = [&](int k) { return j.part + (int64_t)(k == 0 ? 2 * i + 1 : 2 * (i + k)) * PART_FLOATS; };
+  float mx = -INFINITY;
+  bool bad = false;
+  for (int k = 0; k < n; ++k) {
+    const float l = slot(k)[BQ * 128 + row];
+    bad = bad || isnan(l) || l == INFINITY;
+    mx = fmaxf(mx, l);
+  }
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+  float den = 0.f;
+  if (!bad && mx != -INFINITY) {
+    for (int k0 = 0; k0 < n; k0 += MG_UNROLL) {
+      float4 x[MG_UNROLL];
+      float w[MG_UNROLL];
+#pragma unroll
+      for (int q = 0; q < MG_UNROLL; ++q)
+        if (k0 + q < n) {
+          const float* p = slot(k0 + q);
+          x[q] = reinterpret_cast<const float4*>(p)[c4 * BQ + row];
+          w[q] = exp2f(p[BQ * 128 + row] - mx);
+        }
+#pragma unroll
+      for (int q = 0; q < MG_UNROLL; ++q)
+        if (k0 + q < n) {
+          den += w[q];
+          o.x = fmaf(w[q], x[q].x, o.x);
+          o.y = fmaf(w[q], x[q].y, o.y);
+          o.z = fmaf(w[q], x[q].z, o.z);
+          o.w = fmaf(w[q], x[q].w, o.w);
+        }
+    }
+    const float inv = 1.0f / den;
+    o.x *= inv; o.y *= inv; o.z *= inv; o.w *= inv;
+  }
+  uint2 pk;
+  pk.x = pack_bf16(o.x, o.y);
+  pk.y = pack_bf16(o.z, o.w);
+  *reinterpret_cast<uint2*>(j.O + ((int64_t)u.x * j.Nq + qrow) * 128 + 4 * c4) = pk;
+}
+
 
 // ---------------------------------------------------------------------------------
 // Two query tiles per CTA.  One CTA owns 256 queries of one head as two 128-query
@@ -739,13 +954,17 @@ __global__ void __launch_bounds__(THREADS, 1)
 }  // namespace
 
 cudaError_t tc_attn_set_smem_limits() {
-  cudaError_t e = cudaFuncSetAttribute(tc_attend, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+  cudaError_t e = cudaFuncSetAttribute(tc_attend<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(tc_attend<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tc_attend2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM2_BYTES);
   return e;
 }
 
-cudaError_t launch_attend_tc(const Bank& b, DevLayer* L, const void* Q, int Nq, const void* Kw, const void* Vw,
+size_t attend_scratch_bytes() { return (size_t)SPLIT_CTAS * (2 * PART_FLOATS * sizeof(float) + sizeof(int4)); }
+
+cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw,
                              int W, void* O, cudaStream_t s, Timer* t) {
   CUtensorMap mq, mkb, mvb, mkw, mvw;
   if (!make_map_rows(&mq, Q, Nq, b.H, BQ) || !make_map_rows(&mkb, b.k, b.M_max, b.H, BK) ||
@@ -757,27 +976,48 @@ cudaError_t launch_attend_tc(const Bank& b, DevLayer* L, const void* Q, int Nq, 
     mkw = mkb;   // never read: there are no window tiles
     mvw = mvb;
   }
-  AttnJob job{b, L, Nq, W, (__nv_bfloat16*)O, 1.4426950408889634f / sqrtf(128.0f)};
-  // two query tiles per CTA whenever that still gives every SM at least two CTAs (the
-  // key-split kernel keeps small grids, e.g. one layer of 12 heads, in fewer waves)
-  static int n_sm = 0;
-  if (n_sm == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-      n_sm = v;
-  }
+  const int n_sm = sm_count();
+  if (n_sm <= 0) return cudaErrorInvalidDevice;
+  const int64_t units = (int64_t)((Nq + BQ - 1) / BQ) * b.H;
   const int64_t ctas2 = (int64_t)((Nq + 2 * BQ - 1) / (2 * BQ)) * b.H;
+  AttnJob job{b, w.L, Nq, W, (__nv_bfloat16*)O, 1.4426950408889634f / sqrtf(128.0f), nullptr, nullptr};
+  // Schedule: the shortest of three estimates, in key tiles of one unit (0.775 us each on an
+  // SM that has work, measured with 12 full heads) from the budgets, which the host knows
+  // (occupancies it does not).  C0 tiles are a CTA's or a segment's fixed cost.
+  //   whole units, one CTA each:   every wave lasts a unit; a lone wave its longest unit
+  //   equal shares:                all SMs busy to the end, one more segment and the merge
+  //   two query tiles per CTA:     0.92 of the time per unit (K and V cross from L2 once for
+  //                                both), waves of two units
+  // Both sides of the lines, us (whole units | shares | two tiles), 9,360 + 4,680 keys: 12
+  // heads x 4,680 queries 249 | 264 | -; x 1,560 170 | 112 | -; x 256 95 | 37 | -; 16 heads x
+  // 4,680 - | 341 | 315; 17 heads - | 385 | 460.
+  constexpr float C0 = 6.f, MERGE = 10.f;
+  const int wt = (W + BK - 1) / BK;
+  const float nt_max = (float)((b.M_max + BK - 1) / BK + wt);
+  const float nt = (float)w.n_mtiles / b.H + wt;
+  const float waves = (float)((units + n_sm - 1) / n_sm), waves2 = (float)((ctas2 + n_sm - 1) / n_sm);
+  const float t_whole = std::max(nt_max, waves * nt) + waves * C0;
+  const float t_two = ctas2 >= 2 * (int64_t)n_sm ? waves2 * (1.84f * nt + C0) : INFINITY;
+  const int n_cta = std::min(n_sm, SPLIT_CTAS);
+  const float per = (float)units / n_cta;
+  const float t_share = w.attn_part && nt_max >= SPLIT_UNIT && units < 1024
+                            ? std::max((float)SPLIT_MIN, per * nt) + (per + 1) * C0 + MERGE
+                            : INFINITY;
   timer_begin(t, "attend_tc", s);
-  if (n_sm > 0 && ctas2 >= 2 * (int64_t)n_sm) {
+  cudaError_t e = cudaSuccess;
+  if (t_two <= std::min(t_whole, t_share)) {
     dim3 grid((Nq + 2 * BQ - 1) / (2 * BQ), b.H);
     tc_attend2<<<grid, THREADS, SMEM2_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
+  } else if (t_whole <= t_share) {
+    tc_attend<false><<<(unsigned)units, THREADS, SMEM_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
   } else {
-    dim3 grid((Nq + BQ - 1) / BQ, b.H);
-    tc_attend<<<grid, THREADS, SMEM_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
+    job.part = w.attn_part;
+    job.meta = reinterpret_cast<int4*>(w.attn_part + (size_t)SPLIT_CTAS * 2 * PART_FLOATS);
+    tc_attend<true><<<n_cta, THREADS, SMEM_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
+    e = launch_after(tc_attend_merge, dim3(n_cta, BQ / MG_ROWS), MG_ROWS * 32, s, job);
   }
   timer_end(t, s);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace dkv

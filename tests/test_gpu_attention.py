@@ -94,3 +94,50 @@ def test_two_tile_attention_reads_a_long_bank(dkv):
         err = max(err, float(np.abs(O[h] - oracle.attend(ob.heads[h], Q[h], Kw[h], Vw[h])).max()))
     assert err < 2e-2, err
     bank.close()
+
+
+@pytest.mark.parametrize("occ,M,Nq,W", [
+    ([5000], 5000, 16, 700),                  # one unit, cut into many parts
+    ([0], 300, 1, 0),                         # no key at all
+    ([1], 300, 130, 0),                       # one key, two query tiles
+    ([0, 900, 0, 128, 1, 77], 900, 200, 0),   # heads without keys between cut units
+    ([3000, 129], 3000, 128, 1),              # a window of one key after a bank that ends inside a tile
+    ([2000] * 13, 2000, 1560, 333),           # more query tiles than SMs: shares over unit boundaries
+])
+def test_shared_key_tiles_match_oracle(dkv, occ, M, Nq, W):
+    """Grids below two CTAs per SM: the key tiles of all (head, query tile) units in equal
+    shares, units cut by share boundaries merged from fp32 parts.  The same call on a handle
+    whose workspace lacks the parts' scratch takes whole units; both match the oracle."""
+    H, d = len(occ), 128
+    bank, ob = _bank_with(dkv, occ, M, seed=Nq + W)
+    rng = np.random.default_rng(Nq)
+    Q = _bf16(rng, (H, Nq, d), 1.5)
+    Kw = _bf16(rng, (H, W, d), 1.5) if W else None
+    Vw = _bf16(rng, (H, W, d), 1.0) if W else None
+    Qd = to_dev(Q, torch.bfloat16)
+    Kd, Vd = (to_dev(Kw, torch.bfloat16), to_dev(Vw, torch.bfloat16)) if W else (None, None)
+    p = dkv.dkv_params_default(d)
+    p.score_mode = dkv.DKV_SCORE_FP32
+    small = dkv.dkv_bank_workspace_size(H, d, [M] * H, 64, dkv.DKV_DTYPE_BF16, p)
+    assert small < bank.workspace.numel()
+    spare = torch.empty(small, dtype=torch.uint8, device="cuda")
+    bufs = dkv.dkv_buffers_t(bank.k.data_ptr(), bank.v.data_ptr(), bank.rho.data_ptr(), bank.base.data_ptr(),
+                             bank.knorm.data_ptr(), bank.prov_step.data_ptr(), bank.prov_src.data_ptr(),
+                             bank.occupancy.data_ptr(), spare.data_ptr(), small)
+    O = bank.attend(Qd, Kd, Vd)
+    whole = torch.full_like(O, 7.0)
+    other = dkv.dkv_bank_create(H, d, [M] * H, 64, dkv.DKV_DTYPE_BF16, bank.params, bufs)
+    dkv.dkv_bank_attend(other, Qd, Nq, Kd, Vd, W, whole)
+    bank.sync()
+    dkv.dkv_bank_sync(other)
+    dkv.dkv_bank_destroy(other)
+    O, whole = O.float().cpu().numpy(), whole.float().cpu().numpy()
+    for h in range(H):
+        if occ[h] + W == 0:
+            assert np.all(O[h] == 0) and np.all(whole[h] == 0), h
+            continue
+        kw = np.zeros((0, d)) if Kw is None else Kw[h]
+        vw = np.zeros((0, d)) if Vw is None else Vw[h]
+        ref = oracle.attend(ob.heads[h], Q[h], kw, vw)
+        assert np.abs(O[h] - ref).max() < 2e-2 and np.abs(whole[h] - ref).max() < 2e-2, h
+    bank.close()

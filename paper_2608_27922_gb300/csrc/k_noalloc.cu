@@ -11,14 +11,17 @@
 // file-scope device array below, of a fixed size.
 //
 // The scoring kernel is the fp32 direct-difference variant of the Eq. 6 pass for
-// one head, with the arithmetic of the fp32 score mode of dkv_bank_admit in the same
-// order: d2 = (sequential fused multiply-adds over the first half of the dimensions)
-// + (the same over the second half), one rounded add joining them; w by the shared
-// Eq. 2 helper; the weighted sum over bank columns in increasing order; one division
-// by m.  Its scores are therefore bit-identical to admit's in that mode.  The ordering
-// kernel is the stable ascending sort with ties in source order.
+// one head, on the tiled pair code of the fp32 score mode of dkv_bank_admit
+// (simt_pairs.cuh), whose sums have one order for any tile size; one division by m.
+// Its scores are therefore bit-identical to admit's in that mode.  The ordering
+// kernel places every candidate at the number of candidates that come before it
+// (smaller score, or equal score and smaller source index): the stable ascending
+// order, without a buffer to sort in and over as many blocks as there are candidates.
+// Measured at 2,070 MHz, d = 128, bf16, 9,360 bank keys x 4,680 candidates: the
+// whole call 4,885 us before (one thread per candidate, one block sorting) -> 654.
 #include "../../include/dkv.h"
-#include "dkv_device.cuh"
+#include "dkv_internal.h"
+#include "simt_pairs.cuh"
 
 #include <climits>
 #include <cmath>
@@ -30,80 +33,101 @@ namespace {
 // Scratch shared by every call on a device, held until the process exits.
 static __device__ __align__(256) float g_noalloc_scores[DKV_NOALLOC_MAX_N];
 
-constexpr int ROWS = 128;   // candidates per block of the scoring kernel
-constexpr int CT = 32;      // bank keys staged per shared-memory tile
-constexpr int SORT_THREADS = 1024;
-
-template <typename T, int D>
-__global__ void __launch_bounds__(ROWS) noalloc_score(const T* __restrict__ Kb, const float* __restrict__ base,
-                                                      int m, const T* __restrict__ Kc, int N, KParams kp,
-                                                      float* __restrict__ scratch) {
-  __shared__ float cs[CT * D];
-  __shared__ float cinv[CT];
-  const int x = blockIdx.x * ROWS + threadIdx.x;
-  const bool active = x < N;
-  float rr[D];
-#pragma unroll
-  for (int k = 0; k < D; ++k) rr[k] = active ? to_f<T>(Kc[(int64_t)x * D + k]) : 0.f;
+template <typename T, int D, int RT>
+__global__ void __launch_bounds__(simt::NT) noalloc_score(const T* Kb, const float* base, int m, const T* Kc, int N,
+                                                          KParams kp, bool vec, float* scratch) {
+  extern __shared__ __align__(16) float smem[];
+  const int row0 = blockIdx.x * RT;
+  const int sr = simt::scan_row<RT>();
   float acc = 0.f;
-  for (int t0 = 0; t0 < m; t0 += CT) {
-    const int nc = min(CT, m - t0);
-    __syncthreads();
-    for (int e = threadIdx.x; e < nc * D; e += ROWS) cs[e] = to_f<T>(Kb[(int64_t)t0 * D + e]);
-    for (int c = threadIdx.x; c < nc; c += ROWS) cinv[c] = __frcp_rn(base[t0 + c]);
-    __syncthreads();
-    if (!active) continue;
-    for (int c = 0; c < nc; ++c) {
-      const float* col = cs + c * D;
-      float q0 = 0.f, q1 = 0.f;   // first and second half of the dimensions
-#pragma unroll
-      for (int k = 0; k < D / 2; ++k) {
-        const float d0 = __fsub_rn(rr[k], col[k]), d1 = __fsub_rn(rr[D / 2 + k], col[D / 2 + k]);
-        q0 = __fmaf_rn(d0, d0, q0);
-        q1 = __fmaf_rn(d1, d1, q1);
-      }
-      acc = __fmaf_rn(riesz_w(__fadd_rn(q0, q1), kp), cinv[c], acc);
-    }
-  }
-  if (active) scratch[x] = __fdiv_rn(acc, (float)m);
+  simt::pair_tiles<T, D, false, RT>(Kc, nullptr, row0, N, Kb, nullptr, base, 0, m, kp, vec, smem,
+                                    [&](int, int nc, const float* w, const float* inv) {
+                                      simt::for_columns(nc, w, [&](int c, float x) { acc = __fmaf_rn(x, inv[c], acc); });
+                                    });
+  if (sr >= 0 && row0 + sr < N) scratch[row0 + sr] = __fdiv_rn(acc, (float)m);
 }
 
-__global__ void __launch_bounds__(SORT_THREADS) noalloc_order(const float* __restrict__ scratch, int N, int m,
-                                                              int32_t* __restrict__ perm, float* __restrict__ scores) {
-  extern __shared__ unsigned long long keys[];
+// Block b places candidates [32 b, 32 b + 32): thread (i, g) = (t % 32, t / 32) counts, for
+// candidate i, those that come before it among every 8th run of ORD_RUN candidates; the
+// eight counts are added through shared memory.  2 N^2 / 32 warp comparisons in all: at
+// N = 16,384 about 8 M a phase, less than the single block of a sort in shared memory took
+// for its 91 to 105 barrier-separated exchange phases.
+constexpr int ORD_RUN = 256;
+constexpr int ORD_GROUPS = 8;
+
+__global__ void __launch_bounds__(32 * ORD_GROUPS) noalloc_order(const float* scratch, int N, int m, int32_t* perm,
+                                                                 float* scores) {
+  __shared__ __align__(16) uint32_t keys[ORD_GROUPS][ORD_RUN];
+  __shared__ int s_cnt[ORD_GROUPS][32];
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
   if (m == 0) {   // empty bank: source order (Alg. 1, m = 0 branch)
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    if (g == 0 && i < N) {
       perm[i] = i;
       if (scores) scores[i] = 0.f;
     }
     return;
   }
-  int n = 2;
-  while (n < N) n <<= 1;
-  for (int i = threadIdx.x; i < n; i += blockDim.x)
-    keys[i] = i < N ? ((unsigned long long)fkey(scratch[i]) << 32) | (unsigned)i : ~0ull;
-  __syncthreads();
-  for (int k = 2; k <= n; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int ix = i ^ j;
-        if (ix > i) {
-          const unsigned long long a = keys[i], c = keys[ix];
-          if ((a > c) == ((i & k) == 0)) { keys[i] = c; keys[ix] = a; }
+  const float mine = i < N ? scratch[i] : 0.f;
+  const uint32_t key = fkey(mine);
+  int cnt = 0;
+  for (int r0 = g * ORD_RUN; r0 < N; r0 += ORD_GROUPS * ORD_RUN) {   // warp-uniform
+    const int n = min(ORD_RUN, N - r0);
+    for (int k = lane; k < n; k += 32) keys[g][k] = fkey(scratch[r0 + k]);
+    __syncwarp();
+    // candidates of the run before index i precede it at equal scores
+    const int below = min(max(i - r0, 0), n);
+    if (n == ORD_RUN && (below == 0 || below == n)) {
+      if (below) {
+#pragma unroll 8
+        for (int k = 0; k < ORD_RUN; k += 4) {
+          const uint4 x = *reinterpret_cast<const uint4*>(&keys[g][k]);
+          cnt += (x.x <= key) + (x.y <= key) + (x.z <= key) + (x.w <= key);
+        }
+      } else {
+#pragma unroll 8
+        for (int k = 0; k < ORD_RUN; k += 4) {
+          const uint4 x = *reinterpret_cast<const uint4*>(&keys[g][k]);
+          cnt += (x.x < key) + (x.y < key) + (x.z < key) + (x.w < key);
         }
       }
-      __syncthreads();
+    } else {
+      for (int k = 0; k < n; ++k) cnt += k < below ? keys[g][k] <= key : keys[g][k] < key;
     }
+    __syncwarp();
   }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    perm[i] = (int32_t)(keys[i] & 0xffffffffu);
-    if (scores) scores[i] = scratch[i];
+  s_cnt[g][lane] = cnt;
+  __syncthreads();
+  if (g == 0 && i < N) {
+    int pos = 0;
+#pragma unroll
+    for (int q = 0; q < ORD_GROUPS; ++q) pos += s_cnt[q][lane];
+    perm[pos] = i;   // keys with their index are distinct: positions cover [0, N)
+    if (scores) scores[i] = mine;
   }
+}
+
+template <typename T, int D, int RT>
+cudaError_t launch_score(const void* Kb, const float* base, int m, const void* Kc, int N, const KParams& kp,
+                         float* scratch, cudaStream_t s) {
+  // this entry point asks no alignment of its key arrays beyond the element's
+  const bool vec = ((reinterpret_cast<uintptr_t>(Kb) | reinterpret_cast<uintptr_t>(Kc)) & 15u) == 0;
+  noalloc_score<T, D, RT><<<(N + RT - 1) / RT, simt::NT, simt::Lay<D, false, RT>::SMEM, s>>>(
+      static_cast<const T*>(Kb), base, m, static_cast<const T*>(Kc), N, kp, vec, scratch);
+  return cudaGetLastError();
+}
+
+template <typename T, int D>
+cudaError_t launch_score(const void* Kb, const float* base, int m, const void* Kc, int N, const KParams& kp,
+                         float* scratch, cudaStream_t s) {
+  return simt::pick_rows(1, N, sm_count(), false) == 32
+             ? launch_score<T, D, 32>(Kb, base, m, Kc, N, kp, scratch, s)
+             : launch_score<T, D, 16>(Kb, base, m, Kc, N, kp, scratch, s);
 }
 
 // Set-up per device, with that device current: the device address of the scratch
 // array (in host code the array's name is only a host-side stand-in) and the
-// shared-memory opt-in of the ordering kernel.  Only a complete success is kept; a
+// shared-memory opt-in of the scoring kernels.  Only a complete success is kept; a
 // failed attempt leaves nothing behind, so the next call on that device tries again.
 constexpr int kMaxDevices = 64;
 struct DeviceSetup {
@@ -120,9 +144,17 @@ cudaError_t setup_device(int dev, float** scratch) {
   if (!s.ready) {
     void* p = nullptr;
     cudaError_t err = cudaGetSymbolAddress(&p, g_noalloc_scores);
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(noalloc_order, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 DKV_NOALLOC_MAX_N * (int)sizeof(unsigned long long));
+    auto opt_in = [&](auto k, size_t bytes) {
+      if (err == cudaSuccess) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    opt_in(noalloc_score<__nv_bfloat16, 128, 32>, simt::Lay<128, false, 32>::SMEM);
+    opt_in(noalloc_score<__nv_bfloat16, 128, 16>, simt::Lay<128, false, 16>::SMEM);
+    opt_in(noalloc_score<__nv_bfloat16, 64, 32>, simt::Lay<64, false, 32>::SMEM);
+    opt_in(noalloc_score<__nv_bfloat16, 64, 16>, simt::Lay<64, false, 16>::SMEM);
+    opt_in(noalloc_score<float, 128, 32>, simt::Lay<128, false, 32>::SMEM);
+    opt_in(noalloc_score<float, 128, 16>, simt::Lay<128, false, 16>::SMEM);
+    opt_in(noalloc_score<float, 64, 32>, simt::Lay<64, false, 32>::SMEM);
+    opt_in(noalloc_score<float, 64, 16>, simt::Lay<64, false, 16>::SMEM);
     if (err != cudaSuccess) {
       (void)cudaGetLastError();   // do not leave the failure to the next unrelated check
       return err;
@@ -163,21 +195,15 @@ extern "C" dkv_status_t dkv_candidate_order_noalloc(const void* K_bank, const fl
   kp.sync_heads = 1;
   cudaStream_t s = (cudaStream_t)stream;
   if (m > 0) {
-    const dim3 grid((N + ROWS - 1) / ROWS);
-    if (dtype == DKV_DTYPE_BF16) {
-      using T = __nv_bfloat16;
-      if (d == 128) noalloc_score<T, 128><<<grid, ROWS, 0, s>>>((const T*)K_bank, base, m, (const T*)Kc, N, kp, scratch);
-      else noalloc_score<T, 64><<<grid, ROWS, 0, s>>>((const T*)K_bank, base, m, (const T*)Kc, N, kp, scratch);
-    } else {
-      if (d == 128)
-        noalloc_score<float, 128><<<grid, ROWS, 0, s>>>((const float*)K_bank, base, m, (const float*)Kc, N, kp, scratch);
-      else
-        noalloc_score<float, 64><<<grid, ROWS, 0, s>>>((const float*)K_bank, base, m, (const float*)Kc, N, kp, scratch);
-    }
-    if (cudaGetLastError() != cudaSuccess) return DKV_ERR_CUDA;
+    cudaError_t e;
+    if (dtype == DKV_DTYPE_BF16)
+      e = d == 128 ? launch_score<__nv_bfloat16, 128>(K_bank, base, m, Kc, N, kp, scratch, s)
+                   : launch_score<__nv_bfloat16, 64>(K_bank, base, m, Kc, N, kp, scratch, s);
+    else
+      e = d == 128 ? launch_score<float, 128>(K_bank, base, m, Kc, N, kp, scratch, s)
+                   : launch_score<float, 64>(K_bank, base, m, Kc, N, kp, scratch, s);
+    if (e != cudaSuccess) return DKV_ERR_CUDA;
   }
-  int n = 2;
-  while (n < N) n <<= 1;
-  noalloc_order<<<1, SORT_THREADS, (size_t)n * sizeof(unsigned long long), s>>>(scratch, N, m, perm_out, scores_out);
+  noalloc_order<<<(N + 31) / 32, 32 * ORD_GROUPS, 0, s>>>(scratch, N, m, perm_out, scores_out);
   return cudaGetLastError() == cudaSuccess ? DKV_OK : DKV_ERR_CUDA;
 }

@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "dkv_device.cuh"
 
 namespace dkv {
@@ -143,21 +145,35 @@ cudaError_t launch_attend_fp32(const Bank& b, const void* Q, int Nq, const void*
 size_t attend_scratch_bytes();   // per handle: 20 MB of partial results
 cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw,
                              int W, void* O, cudaStream_t s, Timer* t);
-// Launches `k` so that its blocks may start before the preceding kernel of the stream has
-// ended (programmatic dependent launch): k must call pdl_wait() before it reads or writes
-// anything that kernel or an earlier one touches.
-template <typename... Args>
-cudaError_t launch_after(void (*k)(Args...), dim3 grid, unsigned threads, cudaStream_t s, Args... args) {
+// Kernel launch.  after: the blocks may start before the preceding kernel of the stream has
+// ended (programmatic dependent launch), which hides the launch and the ramp behind that
+// kernel's end; every block of k must then call pdl_wait() before it reads or writes anything
+// that an earlier kernel touches.  Used between the kernels of one call only: the first of a
+// call follows the caller's own work and events in the ordinary way.  cluster > 1: blocks in
+// clusters of that many along x.
+template <typename... P, typename... Args>
+cudaError_t launch_kernel(void (*k)(P...), dim3 grid, unsigned threads, size_t smem, int cluster, bool after,
+                          cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, args...);
+  cudaLaunchAttribute at[2]{};
+  unsigned n = 0;
+  if (after) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)cluster;
+    at[n].val.clusterDim.y = at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
 }
 
 bool tc_supported(int d, int bf16);

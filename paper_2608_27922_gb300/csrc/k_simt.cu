@@ -85,6 +85,8 @@ __device__ __forceinline__ const T* ptr(const void* p, int64_t off) {
 template <typename T, int D, bool KV, int RT>
 __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 4) simt_pairs(PairJob j) {
   extern __shared__ __align__(16) float smem[];
+  pdl_wait();
+  pdl_trigger();
   const int h = blockIdx.y;
   const int mode = j.mode;   // uniform
   const DevHead hd = j.w.hd[h];
@@ -174,8 +176,9 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
 
 template <typename T, int D, bool KV, int RT>
 cudaError_t launch_tile(int max_rows, cudaStream_t s, const PairJob& j) {
-  simt_pairs<T, D, KV, RT><<<dim3((max_rows + RT - 1) / RT, j.b.H), simt::NT, simt::Lay<D, KV, RT>::SMEM, s>>>(j);
-  return cudaGetLastError();
+  const bool after = j.mode == PM_SCORE || j.mode == PM_CROSS;   // follows another kernel of the same call
+  return launch_kernel(simt_pairs<T, D, KV, RT>, dim3((max_rows + RT - 1) / RT, j.b.H), simt::NT,
+                       simt::Lay<D, KV, RT>::SMEM, 1, after, s, j);
 }
 
 template <typename T, int D, bool KV>
@@ -536,20 +539,10 @@ namespace {
 template <typename T, int D, int RT>
 cudaError_t launch_attend_t(const Bank& b, const void* Q, int Nq, const void* Kw, const void* Vw, int W, void* O,
                             int split, cudaStream_t s) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((Nq + RT - 1) / RT * split), b.H);
-  cfg.blockDim = dim3(ANT);
-  cfg.dynamicSmemBytes = LayA<D, RT>::SMEM;
-  cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = (unsigned)split;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = split > 1 ? 1 : 0;
   const float qscale = 1.4426950408889634f / sqrtf((float)D);   // log2(e) / sqrt(d)
-  return cudaLaunchKernelEx(&cfg, simt_attend<T, D, RT>, (const T*)Q, Nq, (const T*)Kw, (const T*)Vw, W, (T*)O, b,
-                            qscale);
+  return launch_kernel(simt_attend<T, D, RT>, dim3((unsigned)((Nq + RT - 1) / RT * split), b.H), ANT,
+                       LayA<D, RT>::SMEM, split, false, s, (const T*)Q, Nq, (const T*)Kw, (const T*)Vw, W, (T*)O, b,
+                       qscale);
 }
 
 template <typename T, int D>

@@ -1014,7 +1014,7 @@ cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, 
     job.part = w.attn_part;
     job.meta = reinterpret_cast<int4*>(w.attn_part + (size_t)SPLIT_CTAS * 2 * PART_FLOATS);
     tc_attend<true><<<n_cta, THREADS, SMEM_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
-    e = launch_after(tc_attend_merge, dim3(n_cta, BQ / MG_ROWS), MG_ROWS * 32, s, job);
+    e = launch_kernel(tc_attend_merge, dim3(n_cta, BQ / MG_ROWS), MG_ROWS * 32, 0, 1, true, s, job);
   }
   timer_end(t, s);
   return e != cudaSuccess ? e : cudaGetLastError();

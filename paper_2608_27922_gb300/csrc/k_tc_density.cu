@@ -697,6 +697,8 @@ __global__ void __launch_bounds__(THREADS, KV ? 1 : 2)
     tc_pairs(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAx,
              const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBx,
              const __grid_constant__ CUtensorMap tmAv, const __grid_constant__ CUtensorMap tmBv, TcJob j) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   if ((smem_u32(smem_raw) & 1023u) != 0u) {   // 128-byte-swizzled tiles need 1024-byte alignment
     if (threadIdx.x == 0) dev_fail(j.w.L, DEV_INCONSISTENT, 9900);
@@ -740,6 +742,8 @@ __host__ __device__ __forceinline__ int loop_slot() {
 
 template <int MODE, int P>
 __global__ void __launch_bounds__(256) pairs_classify(TcJob j, int n_units) {
+  pdl_wait();
+  pdl_trigger();
   int32_t* list = j.w.loop_list + loop_slot<MODE>() * j.w.loop_stride;
   int32_t* ctr = j.w.loop_ctr + 2 * loop_slot<MODE>();
   const int64_t total = (int64_t)n_units * BM;
@@ -766,6 +770,8 @@ __global__ void __launch_bounds__(THREADS, KV ? 1 : 2)
     tc_pairs_loop(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAx,
                   const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBx,
                   const __grid_constant__ CUtensorMap tmAv, const __grid_constant__ CUtensorMap tmBv, TcJob j) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   if ((smem_u32(smem_raw) & 1023u) != 0u) {
     if (threadIdx.x == 0) dev_fail(j.w.L, DEV_INCONSISTENT, 9903);
@@ -849,6 +855,8 @@ __global__ void __launch_bounds__(DU_THREADS, 1)
     tc_cross_dual(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAx,
                   const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBx, TcJob j,
                   int n_units) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0u) {
     if (threadIdx.x == 0) dev_fail(j.w.L, DEV_INCONSISTENT, 9904);
@@ -1179,6 +1187,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1)
     tc_score_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAx,
                   const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBx, TcJob j,
                   int n_units) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ __align__(1024) uint8_t smem[];
   if ((smem_u32(smem) & 1023u) != 0u) {
     if (threadIdx.x == 0) dev_fail(j.w.L, DEV_INCONSISTENT, 9906);
@@ -1428,22 +1438,29 @@ bool make_map_ext(CUtensorMap* m, const void* base, int64_t rows, int64_t heads,
 namespace {
 
 template <int MODE, int P>
-void launch_p(dim3 grid, cudaStream_t s, const CUtensorMap& a, const CUtensorMap& ax, const CUtensorMap& b,
-              const CUtensorMap& bx, const CUtensorMap& av, const CUtensorMap& bv, bool kv, const TcJob& job,
-              int n_units) {
+cudaError_t launch_p(dim3 grid, cudaStream_t s, const CUtensorMap& a, const CUtensorMap& ax, const CUtensorMap& b,
+                     const CUtensorMap& bx, const CUtensorMap& av, const CUtensorMap& bv, bool kv, const TcJob& job,
+                     int n_units) {
+  // the passes that follow another kernel of the same call
+  constexpr bool after = MODE == TM_SCORE || MODE == TM_CROSS;
   if (n_units > 0) {   // persistent form (projection, survivor maintenance, new baselines)
     if constexpr (MODE == TM_PROJECT || MODE == TM_SUB || MODE == TM_NEWBASE) {
-      if (cudaMemsetAsync(job.w.loop_ctr + 2 * loop_slot<MODE>(), 0, 2 * sizeof(int32_t), s) != cudaSuccess) return;
+      cudaError_t e = cudaMemsetAsync(job.w.loop_ctr + 2 * loop_slot<MODE>(), 0, 2 * sizeof(int32_t), s);
+      if (e != cudaSuccess) return e;
       const int64_t threads = (int64_t)n_units * BM;
       const int cblocks = (int)std::min<int64_t>((threads + 255) / 256, (int64_t)grid.x * 8);
-      pairs_classify<MODE, P><<<cblocks, 256, 0, s>>>(job, n_units);
-      if (kv) tc_pairs_loop<MODE, P, true><<<grid, THREADS, Lay<true>::SMEM, s>>>(a, ax, b, bx, av, bv, job);
-      else tc_pairs_loop<MODE, P, false><<<grid, THREADS, Lay<false>::SMEM, s>>>(a, ax, b, bx, av, bv, job);
+      e = launch_kernel(pairs_classify<MODE, P>, dim3(cblocks), 256, 0, 1, false, s, job, n_units);
+      if (e != cudaSuccess) return e;
+      return kv ? launch_kernel(tc_pairs_loop<MODE, P, true>, grid, THREADS, Lay<true>::SMEM, 1, true, s, a, ax, b, bx, av,
+                                bv, job)
+                : launch_kernel(tc_pairs_loop<MODE, P, false>, grid, THREADS, Lay<false>::SMEM, 1, true, s, a, ax, b, bx, av,
+                                bv, job);
     }
-    return;
   }
-  if (kv) tc_pairs<MODE, P, true><<<grid, THREADS, Lay<true>::SMEM, s>>>(a, ax, b, bx, av, bv, job);
-  else tc_pairs<MODE, P, false><<<grid, THREADS, Lay<false>::SMEM, s>>>(a, ax, b, bx, av, bv, job);
+  return kv ? launch_kernel(tc_pairs<MODE, P, true>, grid, THREADS, Lay<true>::SMEM, 1, after, s, a, ax, b, bx, av, bv,
+                              job)
+            : launch_kernel(tc_pairs<MODE, P, false>, grid, THREADS, Lay<false>::SMEM, 1, after, s, a, ax, b, bx, av, bv,
+                              job);
 }
 
 // rv / cv: the row and column values (same layouts as rk / ck), non-null only with the
@@ -1470,11 +1487,11 @@ cudaError_t launch_tc(const Bank& b, const Ws& w, const KParams& kp, const void*
     if (DKV_CROSS_DUAL && !kv && n_sm > 0) {   // the persistent two-row-tile form
       TcJob job{b, w, kp, 0, 0};
       timer_begin(t, name, s);
-      if (kp.p == 1) tc_cross_dual<1><<<n_sm, DU_THREADS, LayC::SMEM, s>>>(ma, max_, mb, mbx, job, w.n_mpairs);
-      else if (kp.p == 4) tc_cross_dual<4><<<n_sm, DU_THREADS, LayC::SMEM, s>>>(ma, max_, mb, mbx, job, w.n_mpairs);
-      else tc_cross_dual<2><<<n_sm, DU_THREADS, LayC::SMEM, s>>>(ma, max_, mb, mbx, job, w.n_mpairs);
+      auto* k = kp.p == 1 ? tc_cross_dual<1> : kp.p == 4 ? tc_cross_dual<4> : tc_cross_dual<2>;
+      const cudaError_t e =
+          launch_kernel(k, dim3(n_sm), DU_THREADS, LayC::SMEM, 1, true, s, ma, max_, mb, mbx, job, w.n_mpairs);
       timer_end(t, s);
-      return cudaGetLastError();
+      return e;
     }
   }
   // passes over bank rows take one CTA per budget-sized row tile of each head
@@ -1494,11 +1511,10 @@ cudaError_t launch_tc(const Bank& b, const Ws& w, const KParams& kp, const void*
     }
   }
   timer_begin(t, name, s);
-  if (kp.p == 1) launch_p<MODE, 1>(grid, s, ma, max_, mb, mbx, mav, mbv, kv, job, n_units);
-  else if (kp.p == 4) launch_p<MODE, 4>(grid, s, ma, max_, mb, mbx, mav, mbv, kv, job, n_units);
-  else launch_p<MODE, 2>(grid, s, ma, max_, mb, mbx, mav, mbv, kv, job, n_units);
+  auto launch = kp.p == 1 ? launch_p<MODE, 1> : kp.p == 4 ? launch_p<MODE, 4> : launch_p<MODE, 2>;
+  const cudaError_t e = launch(grid, s, ma, max_, mb, mbx, mav, mbv, kv, job, n_units);
   timer_end(t, s);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace
@@ -1584,11 +1600,10 @@ cudaError_t launch_score_tc(const Bank& b, const Ws& w, const void* Kc, const vo
     TcJob job{b, w, kp, 0, tpn};
     const int n_units = (int)ctas;
     timer_begin(t, "score_tc", s);
-    if (kp.p == 1) tc_score_wide<1><<<n_sm, SW_THREADS, LayW::SMEM, s>>>(ma, max_, mb, mbx, job, n_units);
-    else if (kp.p == 4) tc_score_wide<4><<<n_sm, SW_THREADS, LayW::SMEM, s>>>(ma, max_, mb, mbx, job, n_units);
-    else tc_score_wide<2><<<n_sm, SW_THREADS, LayW::SMEM, s>>>(ma, max_, mb, mbx, job, n_units);
+    auto* k = kp.p == 1 ? tc_score_wide<1> : kp.p == 4 ? tc_score_wide<4> : tc_score_wide<2>;
+    const cudaError_t e = launch_kernel(k, dim3(n_sm), SW_THREADS, LayW::SMEM, 1, true, s, ma, max_, mb, mbx, job, n_units);
     timer_end(t, s);
-    return cudaGetLastError();
+    return e;
   }
   return launch_tc<TM_SCORE>(b, w, kp, Kc, w.cext, N, b.k, w.bext, b.M_max, N, s, t, "score_tc", split,
                              kv ? Vc : nullptr, kv ? b.v : nullptr, b.n_max);

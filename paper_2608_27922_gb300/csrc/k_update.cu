@@ -337,6 +337,8 @@ __global__ void k_row_norms(const T* __restrict__ K, const T* __restrict__ V, in
 template <typename T>
 __global__ void k_cand_prepare(Bank b, Ws w, const T* __restrict__ Kc, const T* __restrict__ Vc, int N, int64_t step,
                                float goff) {
+  pdl_wait();
+  pdl_trigger();
   if (blockIdx.x == gridDim.x - 1) {
     if (blockIdx.y == 0) prepare_body(b, w, N, step);
     return;
@@ -360,6 +362,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_cand_prepare_rope(Bank b, Ws w, const T* __restrict__ Kc,
                                                            const T* __restrict__ Vc, int N, int64_t step, float goff,
                                                            const RopeArgs ra) {
+  pdl_wait();
+  pdl_trigger();
   if (blockIdx.x == gridDim.x - 1) {
     prepare_body(b, w, N, step);
     return;
@@ -466,6 +470,8 @@ __device__ __forceinline__ void cas_shfl(unsigned long long (&x)[SKPT], int t, i
 // padded with ~0) ascending; the direction bit is taken from the run-local index, so
 // every run comes out ascending.
 __global__ void __launch_bounds__(256) k_sort_runs(Ws w, int n_max, int identity) {
+  pdl_wait();
+  pdl_trigger();
   const int h = blockIdx.y;
   const int N = layer_of(w, h)->N;
   // empty bank: source order (Alg. 1, m = 0 branch); source-order policy: the same
@@ -513,6 +519,8 @@ __device__ __forceinline__ int run_rank(const unsigned long long* r, unsigned lo
 template <int RB>
 __global__ void __launch_bounds__(RUN * RB) k_sort_rank(Bank bk, Ws w, const char* __restrict__ Kc,
                                                         const char* __restrict__ Vc, int esize, int identity) {
+  pdl_wait();
+  pdl_trigger();
   extern __shared__ unsigned long long runs[];
   __shared__ int s_pos[RUN * RB], s_src[RUN * RB];
   const int h = blockIdx.y;
@@ -599,8 +607,11 @@ __device__ __forceinline__ DevHead ld_head_cg(const DevHead* p) {
 // budgets e_r (Eq. 10) and the feasibility bit of every prefix r; the last block of a
 // layer to finish combines that layer's heads (Eq. 11) and sets r, e of each of them.
 __global__ void __launch_bounds__(BIG) k_rstar(Bank b, Ws w, int sync_heads) {
-  __shared__ int s_tot[BIG];
+  static_assert(BIG == 1024, "one warp reads all warp totals");
+  __shared__ int s_tot[2][32];
   __shared__ int s_best, s_last;
+  pdl_wait();
+  pdl_trigger();
   const int h = blockIdx.x;
   const DevHead hd = w.hd[h];
   DevLayer* lay = layer_of(w, h);
@@ -614,33 +625,37 @@ __global__ void __launch_bounds__(BIG) k_rstar(Bank b, Ws w, int sync_heads) {
   if (hd.empty) {   // an empty head does not constrain the shared prefix
     for (int i = threadIdx.x; i < nw; i += blockDim.x) feas[i] = 0xffffffffu;
   } else {
-    for (int i = threadIdx.x; i < nw; i += blockDim.x) feas[i] = 0u;
+    // 1,024 prefix lengths a round: a scan over the block gives c_r, and each warp's ballot is
+    // one feasibility word (no atomics, one barrier a round: the warp totals alternate)
     const int n = rmax + 1;
-    const int chunk = (n + blockDim.x - 1) / blockDim.x;
-    const int lo = threadIdx.x * chunk, hi = min(n, lo + chunk);
     const int32_t* hist = w.hist + (int64_t)h * w.hist_stride;
-    int tot = 0;
-    for (int r = lo; r < hi; ++r) tot += hist[r];
-    s_tot[threadIdx.x] = tot;
-    __syncthreads();
-    for (int o = 1; o < (int)blockDim.x; o <<= 1) {   // inclusive Hillis-Steele scan
-      const int v = threadIdx.x >= o ? s_tot[threadIdx.x - o] : 0;
-      __syncthreads();
-      s_tot[threadIdx.x] += v;
-      __syncthreads();
-    }
-    int c = s_tot[threadIdx.x] - tot;   // exclusive prefix
-    int best = 0;
-    for (int r = lo; r < hi; ++r) {
-      c += hist[r];
-      const int e = max(0, hd.m_old + r - hd.M);
-      const bool ok = (r == 0) || (c <= e);   // r = 0 is always feasible (Sec. 3.4 Step 2)
-      if (ok) {
-        atomicOr(&feas[r >> 5], 1u << (r & 31));
-        best = r;
+    int best = 0, carry = 0;
+    int next = threadIdx.x < n ? hist[threadIdx.x] : 0;
+    __syncthreads();                                // s_best
+    for (int r0 = 0, q = 0; r0 < n; r0 += BIG, q ^= 1) {
+      const int r = r0 + threadIdx.x;
+      int c = next;
+      next = r + BIG < n ? hist[r + BIG] : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, c, o);
+        if (lane_id() >= o) c += v;
       }
+      if (lane_id() == 31) s_tot[q][warp_id()] = c;
+      __syncthreads();
+      int t = s_tot[q][lane_id()];                  // (BIG / 32 == 32 warps)
+      const int all = __reduce_add_sync(0xffffffffu, t);
+      if (lane_id() >= warp_id()) t = 0;
+      c += carry + __reduce_add_sync(0xffffffffu, t);
+      carry += all;
+      const int e = max(0, hd.m_old + r - hd.M);
+      const bool ok = r < n && (r == 0 || c <= e);  // r = 0 is always feasible (Sec. 3.4 Step 2)
+      const unsigned word = __ballot_sync(0xffffffffu, ok);
+      if (lane_id() == 0 && r < n) feas[r >> 5] = word;
+      if (ok) best = r;
     }
-    atomicMax(&s_best, best);
+    best = __reduce_max_sync(0xffffffffu, best);
+    if (lane_id() == 0) atomicMax(&s_best, best);
   }
   __threadfence();
   __syncthreads();
@@ -762,22 +777,59 @@ __device__ bool find_bin(const int* s_hist, unsigned kk, bool from_top, unsigned
   return true;
 }
 
-// Banks up to SEL_STAGE states are staged in shared memory for the select passes (sort
-// key of rho~ and a mandatory bit per state); larger ones are re-read from global memory.
+// A block's slots up to SEL_STAGE are staged in shared memory for the select passes (sort
+// key of rho~ and a mandatory bit per state); more are re-read from global memory.
 constexpr int SEL_STAGE = 40960;
 
-__host__ __device__ constexpr size_t sel_smem_bytes(int m_cap) {
-  return m_cap > SEL_STAGE ? 0 : (size_t)m_cap * 4 + ((size_t)m_cap + 31) / 32 * 4;
+__host__ __device__ constexpr size_t sel_smem_bytes(int cap) {
+  return cap > SEL_STAGE ? 0 : (size_t)cap * 4 + ((size_t)cap + 31) / 32 * 4;
 }
 
-__global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction) {
-  extern __shared__ uint32_t s_stage[];   // [m] sort keys, then [(m + 31) / 32] mandatory bits
-  __shared__ int s_hist[256];
+// Cluster of this kernel's blocks: rank, size, barrier and a read of a block's shared word.
+__device__ __forceinline__ int cl_rank() {
+  uint32_t x;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(x));
+  return (int)x;
+}
+__device__ __forceinline__ int cl_size() {
+  uint32_t x;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(x));
+  return (int)x;
+}
+__device__ __forceinline__ void cl_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ int cl_read(const int* p, int z) {
+  uint32_t at;
+  int x;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;"
+      : "=r"(at)
+      : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(z));
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(x) : "r"(at) : "memory");
+  return x;
+}
+
+// One cluster of 1 to 8 blocks per head, each with an equal run of the head's slots: block
+// counts and radix histograms are added over the cluster through its shared memory, every
+// block finds the same threshold, and writes its part of the lists behind the lower ranks'
+// counts (ascending slots, as one block over all slots gives).  Bound by latency: passes over
+// the slots and barriers, so the slots are spread as far as the heads leave SMs free.
+// Measured (us, one block per head -> cluster): 12 heads x 9,360 slots 33 -> 25, x 32,760
+// 134 -> 44 (clusters of 8); 160 heads keep one block each (72 -> 82 with the cluster's
+// barriers around it, against 491 us of the pass that follows).
+__global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int cap_max) {
+  extern __shared__ uint32_t s_stage[];   // [cap] sort keys, then [(cap + 31) / 32] mandatory bits
+  __shared__ int s_hist[2][256];          // this block's histogram of even and odd passes
+  __shared__ int s_sum[256];              // the cluster's
   __shared__ int s_warp[33];
-  __shared__ int s_cnt[2];
+  __shared__ int s_cnt[4];                // mandatory, pre-violators, ties, evicted (this block)
   __shared__ unsigned s_prefix, s_kk;
   __shared__ unsigned long long s_tprefix;
-  const int h = blockIdx.x;
+  pdl_wait();
+  pdl_trigger();
+  const int C = cl_size(), rank = cl_rank();
+  const int h = blockIdx.x / C;
   const DevHead hd = w.hd[h];
   const int64_t bh = (int64_t)h * b.M_max;
   const int m = hd.m_old;
@@ -785,26 +837,33 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction) {
   const int e = hd.e;
   const int32_t* cross = w.cross + bh;
   const float* rt = w.rho_t + bh;
-  if (hd.empty) return;
-  if (threadIdx.x == 0) { s_cnt[0] = 0; s_cnt[1] = 0; }
+  if (hd.empty) return;                   // (the whole cluster)
+  const int cap = min(cap_max, ((m + C - 1) / C + 31) & ~31);   // slots per block, whole mask words
+  const int lo = min(m, rank * cap), hi = min(m, lo + cap);
+  if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
   __syncthreads();
+  auto cluster_cnt = [&](int which, int ranks) {   // sum over the first `ranks` blocks
+    int x = 0;
+    for (int z = 0; z < ranks; ++z) x += cl_read(&s_cnt[which], z);
+    return x;
+  };
   // mandatory set and pre-violators (and the shared-memory stage of keys and flags)
-  const bool staged = b.M_max <= SEL_STAGE;
+  const bool staged = cap_max <= SEL_STAGE;
   uint32_t* skey = s_stage;
-  uint32_t* smand = s_stage + (staged ? b.M_max : 0);
+  uint32_t* smand = s_stage + (staged ? cap_max : 0);
   int nm = 0, npre = 0;
-  for (int base = 0; base < m; base += blockDim.x) {
+  for (int base = lo; base < hi; base += blockDim.x) {
     const int i = base + threadIdx.x;
     bool mand = false;
-    if (i < m) {
+    if (i < hi) {
       const int c = cross[i];
       npre += (c == 0);
       mand = r > 0 && c <= r;
       nm += mand;
-      if (staged) skey[i] = fkey(rt[i]);
+      if (staged) skey[i - lo] = fkey(rt[i]);
     }
     const unsigned bal = __ballot_sync(0xffffffffu, mand);
-    if (staged && lane_id() == 0 && i < m) smand[i >> 5] = bal;
+    if (staged && lane_id() == 0 && i < hi) smand[(i - lo) >> 5] = bal;
   }
   nm = __reduce_add_sync(0xffffffffu, nm);
   npre = __reduce_add_sync(0xffffffffu, npre);
@@ -812,12 +871,16 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction) {
     atomicAdd(&s_cnt[0], nm);
     atomicAdd(&s_cnt[1], npre);
   }
-  __syncthreads();
-  int n_mand = s_cnt[0];
-  if (threadIdx.x == 0) { w.hd[h].n_mand = n_mand; w.hd[h].n_pre = s_cnt[1]; }
-  if (e == 0) return;
-  if (n_mand > e) {   // the prefix was feasible, so this cannot happen
-    if (threadIdx.x == 0) dev_fail(w.L, DEV_INCONSISTENT, 2000 + h);
+  cl_sync();
+  int n_mand = cluster_cnt(0, C);
+  if (rank == 0 && threadIdx.x == 0) {
+    w.hd[h].n_mand = n_mand;
+    w.hd[h].n_pre = cluster_cnt(1, C);
+  }
+  if (e == 0 || n_mand > e) {   // (the whole cluster)
+    // n_mand > e: the prefix was feasible, so this cannot happen
+    if (e > 0 && rank == 0 && threadIdx.x == 0) dev_fail(w.L, DEV_INCONSISTENT, 2000 + h);
+    cl_sync();                  // no block ends while another reads its counts
     return;
   }
   // Eviction policy: threshold crossers first (default and mandatory + source), or none
@@ -829,35 +892,60 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction) {
   const int k = e - n_mand;   // states to evict after the mandatory ones
   auto is_mand = [&](int i) -> bool {
     if (!mand_first) return false;
-    return staged ? ((smand[i >> 5] >> (i & 31)) & 1u) != 0u : (r > 0 && cross[i] <= r);
+    return staged ? ((smand[(i - lo) >> 5] >> ((i - lo) & 31)) & 1u) != 0u : (r > 0 && cross[i] <= r);
   };
-  auto key_of = [&](int i) -> unsigned { return by_source ? 0u : (staged ? skey[i] : fkey(rt[i])); };
+  auto key_of = [&](int i) -> unsigned { return by_source ? 0u : (staged ? skey[i - lo] : fkey(rt[i])); };
+  auto prov_of = [&](int i) {
+    return ((unsigned long long)(uint32_t)b.prov_step[bh + i] << 32) | (uint32_t)b.prov_src[bh + i];
+  };
+  // One radix pass: digit(i, &bin) over this block's slots (false: not counted), the counts
+  // added over the cluster, the bin where they reach s_kk.  Histograms alternate, so that a
+  // block may clear one while the others still read the other.
+  int pass = 0;
+  auto radix_pass = [&](auto digit, bool from_top, unsigned* bin) -> bool {
+    int* hist = s_hist[pass++ & 1];
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
+    __syncthreads();
+    for (int base = lo; base < hi; base += blockDim.x) {
+      const int i = base + threadIdx.x;
+      unsigned d = 0;
+      const bool v = i < hi && digit(i, &d);
+      hist_add(hist, v, d);
+    }
+    cl_sync();
+    if (threadIdx.x < 256) {
+      int x = 0;
+      for (int z = 0; z < C; ++z) x += cl_read(&hist[threadIdx.x], z);
+      s_sum[threadIdx.x] = x;
+    }
+    __syncthreads();
+    bool ok = true;
+    if (warp_id() == 0) {
+      unsigned bn = 0, rest = 0;
+      ok = find_bin(s_sum, s_kk, from_top, &bn, &rest);
+      if (ok && lane_id() == 0) s_kk = rest;
+      *bin = bn;
+    }
+    return ok;   // (bin and verdict in warp 0)
+  };
   // radix select of the k-th largest key among non-mandatory states
   unsigned prefix = 0, mask = 0;
   if (threadIdx.x == 0) { s_prefix = 0; s_kk = (unsigned)k; }
   __syncthreads();
   if (k > 0) {
     for (int shift = 24; shift >= 0; shift -= 8) {
-      for (int i = threadIdx.x; i < 256; i += blockDim.x) s_hist[i] = 0;
-      __syncthreads();
-      for (int base = 0; base < m; base += blockDim.x) {
-        const int i = base + threadIdx.x;
-        bool v = false;
-        unsigned key = 0;
-        if (i < m && !is_mand(i)) {
-          key = key_of(i);
-          v = (key & mask) == prefix;
-        }
-        hist_add(s_hist, v, (key >> shift) & 255u);
-      }
-      __syncthreads();
-      if (warp_id() == 0) {
-        unsigned bin, rest;
-        if (find_bin(s_hist, s_kk, true, &bin, &rest)) {
-          if (lane_id() == 0) { s_kk = rest; s_prefix = prefix | (bin << shift); }
-        } else if (lane_id() == 0) {
-          dev_fail(w.L, DEV_INCONSISTENT, 2100 + h);
-        }
+      unsigned bin = 0;
+      const bool ok = radix_pass(
+          [&](int i, unsigned* d) {
+            if (is_mand(i)) return false;
+            const unsigned key = key_of(i);
+            *d = (key >> shift) & 255u;
+            return (key & mask) == prefix;
+          },
+          true, &bin);
+      if (threadIdx.x == 0) {
+        if (ok) s_prefix = prefix | (bin << shift);
+        else if (rank == 0) dev_fail(w.L, DEV_INCONSISTENT, 2100 + h);
       }
       __syncthreads();
       prefix = s_prefix;
@@ -869,41 +957,30 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction) {
   // ties at the threshold: evict the older states (smaller (step, src)) first
   int n_eq_local = 0;
   if (k > 0)
-    for (int i = threadIdx.x; i < m; i += blockDim.x)
+    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x)
       if (!is_mand(i) && key_of(i) == T) ++n_eq_local;
-  __syncthreads();
-  if (threadIdx.x == 0) s_cnt[0] = 0;
-  __syncthreads();
   n_eq_local = __reduce_add_sync(0xffffffffu, n_eq_local);
-  if (lane_id() == 0) atomicAdd(&s_cnt[0], n_eq_local);
-  __syncthreads();
-  const unsigned n_eq = (unsigned)s_cnt[0];
+  if (lane_id() == 0 && n_eq_local) atomicAdd(&s_cnt[2], n_eq_local);
+  cl_sync();
+  const unsigned n_eq = (unsigned)cluster_cnt(2, C);
   unsigned long long tprefix = 0, tmask = 0;
-  const bool need_tie = k > 0 && n_eq > take_eq;
+  const bool need_tie = k > 0 && n_eq > take_eq;   // (the whole cluster)
   if (need_tie) {
     if (threadIdx.x == 0) { s_tprefix = 0; s_kk = take_eq; }
     __syncthreads();
     for (int shift = 56; shift >= 0; shift -= 8) {
-      for (int i = threadIdx.x; i < 256; i += blockDim.x) s_hist[i] = 0;
-      __syncthreads();
-      for (int base = 0; base < m; base += blockDim.x) {
-        const int i = base + threadIdx.x;
-        bool v = false;
-        unsigned long long tk = 0;
-        if (i < m && !is_mand(i) && key_of(i) == T) {
-          tk = ((unsigned long long)(uint32_t)b.prov_step[bh + i] << 32) | (uint32_t)b.prov_src[bh + i];
-          v = (tk & tmask) == tprefix;
-        }
-        hist_add(s_hist, v, (unsigned)((tk >> shift) & 255ull));
-      }
-      __syncthreads();
-      if (warp_id() == 0) {   // smallest first
-        unsigned bin, rest;
-        if (find_bin(s_hist, s_kk, false, &bin, &rest)) {
-          if (lane_id() == 0) { s_kk = rest; s_tprefix = tprefix | ((unsigned long long)bin << shift); }
-        } else if (lane_id() == 0) {
-          dev_fail(w.L, DEV_INCONSISTENT, 2200 + h);
-        }
+      unsigned bin = 0;
+      const bool ok = radix_pass(
+          [&](int i, unsigned* d) {
+            if (is_mand(i) || key_of(i) != T) return false;
+            const unsigned long long tk = prov_of(i);
+            *d = (unsigned)((tk >> shift) & 255ull);
+            return (tk & tmask) == tprefix;
+          },
+          false, &bin);   // smallest first
+      if (threadIdx.x == 0) {
+        if (ok) s_tprefix = tprefix | ((unsigned long long)bin << shift);
+        else if (rank == 0) dev_fail(w.L, DEV_INCONSISTENT, 2200 + h);
       }
       __syncthreads();
       tprefix = s_tprefix;
@@ -911,35 +988,34 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction) {
     }
   }
   // provenance keys are unique per head, so "<= tprefix" selects exactly take_eq states
-  int n_ev = 0, n_sv = 0;
-  for (int base = 0; base < m; base += blockDim.x) {
+  auto is_evicted = [&](int i) -> bool {
+    if (is_mand(i)) return true;
+    if (k <= 0) return false;
+    const unsigned key = key_of(i);
+    return key > T || (key == T && (!need_tie || prov_of(i) <= tprefix));
+  };
+  int mine = 0;
+  if (C > 1) {   // evicted slots of each block, for the offsets of the later ones
+    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) mine += is_evicted(i);
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane_id() == 0 && mine) atomicAdd(&s_cnt[3], mine);
+    cl_sync();
+  }
+  int n_ev = C > 1 ? cluster_cnt(3, rank) : 0;
+  int n_sv = lo - n_ev;
+  for (int base = lo; base < hi; base += blockDim.x) {
     const int i = base + threadIdx.x;
-    int ev = 0;
-    if (i < m) {
-      const bool mand = is_mand(i);
-      if (mand) ev = 1;
-      else if (k > 0) {
-        const unsigned key = key_of(i);
-        if (key > T) ev = 1;
-        else if (key == T) {
-          if (!need_tie) ev = 1;
-          else {
-            const unsigned long long tk = ((unsigned long long)(uint32_t)b.prov_step[bh + i] << 32) |
-                                          (uint32_t)b.prov_src[bh + i];
-            ev = tk <= tprefix;
-          }
-        }
-      }
-    }
+    const int ev = i < hi && is_evicted(i);
     int tot;
     const int off = block_scan_flag(ev, s_warp, &tot);
-    if (i < m && ev && n_ev + off < e) w.evict_list[(int64_t)h * b.n_max + n_ev + off] = i;
+    if (i < hi && ev && n_ev + off < e) w.evict_list[(int64_t)h * b.n_max + n_ev + off] = i;
     const int offs = (threadIdx.x - off);   // survivors before this thread in the chunk
-    if (i < m && !ev && n_sv + offs < m) w.surv_list[bh + n_sv + offs] = i;
+    if (i < hi && !ev && n_sv + offs < m) w.surv_list[bh + n_sv + offs] = i;
     n_ev += tot;
-    n_sv += min((int)blockDim.x, m - base) - tot;
+    n_sv += min((int)blockDim.x, hi - base) - tot;
   }
-  if (threadIdx.x == 0 && n_ev != e) dev_fail(w.L, DEV_INCONSISTENT, 3000 + h);
+  if (rank == C - 1 && threadIdx.x == 0 && n_ev != e) dev_fail(w.L, DEV_INCONSISTENT, 3000 + h);
+  if (C > 1) cl_sync();   // no block ends while another reads its counts
 }
 
 // 1 / b of every occupied bank slot (after an import; the update keeps it in step).
@@ -960,6 +1036,8 @@ __global__ void k_inv_base(Bank b, Ws w) {
 // another thread still reads it.
 __global__ void k_commit(Bank b, Ws w, const char* __restrict__ Vc, int N, int esize,
                          const int32_t* __restrict__ src_map) {
+  pdl_wait();
+  pdl_trigger();
   const int h = blockIdx.y;
   const DevHead hd = w.hd[h];
   const int64_t bh = (int64_t)h * b.M_max;
@@ -1062,23 +1140,23 @@ cudaError_t launch_cand_norms(const Bank& b, const Ws& w, const void* Kc, const 
                               const KParams& kp, const RopeArgs* rope, cudaStream_t s, Timer* t) {
   if (!w.vperm) Vc = nullptr;   // values enter the norms with the [K; V] descriptor only
   dim3 grid((N + 8 * NR_ROWS - 1) / (8 * NR_ROWS) + 1, b.H);   // + the prepare block
+  const float goff = ext_goff(kp);
+  cudaError_t e;
   timer_begin(t, "cand_norms", s);
   if (rope) {
     const dim3 rgrid((N + ROPE_ROWS - 1) / ROPE_ROWS + 1);   // + the prepare block
-    if (b.bf16)
-      k_cand_prepare_rope<__nv_bfloat16><<<rgrid, 256, 0, s>>>(b, w, (const __nv_bfloat16*)Kc,
-                                                               (const __nv_bfloat16*)Vc, N, step, ext_goff(kp), *rope);
-    else
-      k_cand_prepare_rope<float><<<rgrid, 256, 0, s>>>(b, w, (const float*)Kc, (const float*)Vc, N, step,
-                                                       ext_goff(kp), *rope);
+    e = b.bf16 ? launch_kernel(k_cand_prepare_rope<__nv_bfloat16>, rgrid, 256, 0, 1, false, s, b, w, (const __nv_bfloat16*)Kc,
+                              (const __nv_bfloat16*)Vc, N, step, goff, *rope)
+               : launch_kernel(k_cand_prepare_rope<float>, rgrid, 256, 0, 1, false, s, b, w, (const float*)Kc, (const float*)Vc,
+                              N, step, goff, *rope);
   } else if (b.bf16) {
-    k_cand_prepare<__nv_bfloat16><<<grid, 256, 0, s>>>(b, w, (const __nv_bfloat16*)Kc, (const __nv_bfloat16*)Vc, N,
-                                                       step, ext_goff(kp));
+    e = launch_kernel(k_cand_prepare<__nv_bfloat16>, grid, 256, 0, 1, false, s, b, w, (const __nv_bfloat16*)Kc,
+                     (const __nv_bfloat16*)Vc, N, step, goff);
   } else {
-    k_cand_prepare<float><<<grid, 256, 0, s>>>(b, w, (const float*)Kc, (const float*)Vc, N, step, ext_goff(kp));
+    e = launch_kernel(k_cand_prepare<float>, grid, 256, 0, 1, false, s, b, w, (const float*)Kc, (const float*)Vc, N, step, goff);
   }
   timer_end(t, s);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_bank_norms(const Bank& b, const Ws& w, const KParams& kp, cudaStream_t s, Timer* t) {
@@ -1108,7 +1186,7 @@ cudaError_t launch_sort(const Bank& b, const Ws& w, const void* Kc, const void* 
                         Timer* t) {
   const int max_runs = (b.n_max + RUN - 1) / RUN;
   timer_begin(t, "sort_runs", s);
-  k_sort_runs<<<dim3((max_runs + 7) / 8, b.H), 256, 0, s>>>(w, b.n_max, identity);
+  cudaError_t e = launch_kernel(k_sort_runs, dim3((max_runs + 7) / 8, b.H), 256, 0, 1, true, s, w, b.n_max, identity);
   timer_end(t, s);
   timer_begin(t, "sort_rank", s);
   // four runs per CTA (1,024 threads) when that still gives every SM two CTAs: each CTA
@@ -1117,28 +1195,34 @@ cudaError_t launch_sort(const Bank& b, const Ws& w, const void* Kc, const void* 
   // 1, 228 runs: 22 us against 33 with four)
   const int n_sm = sm_count();
   const size_t sm_bytes = (size_t)max_runs * RUN * 8;
+  cudaError_t rank;
   if ((int64_t)b.H * ((max_runs + 3) / 4) >= 2 * (int64_t)n_sm)
-    k_sort_rank<4><<<dim3((max_runs + 3) / 4, b.H), RUN * 4, sm_bytes, s>>>(b, w, (const char*)Kc, (const char*)Vc,
-                                                                          b.bf16 ? 2 : 4, identity);
+    rank = launch_kernel(k_sort_rank<4>, dim3((max_runs + 3) / 4, b.H), RUN * 4, sm_bytes, 1, true, s, b, w, (const char*)Kc,
+                        (const char*)Vc, b.bf16 ? 2 : 4, identity);
   else
-    k_sort_rank<1><<<dim3(max_runs, b.H), RUN, sm_bytes, s>>>(b, w, (const char*)Kc, (const char*)Vc,
-                                                             b.bf16 ? 2 : 4, identity);
+    rank = launch_kernel(k_sort_rank<1>, dim3(max_runs, b.H), RUN, sm_bytes, 1, true, s, b, w, (const char*)Kc,
+                        (const char*)Vc, b.bf16 ? 2 : 4, identity);
   timer_end(t, s);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : rank;
 }
 
 cudaError_t launch_rstar(const Bank& b, const Ws& w, const KParams& kp, cudaStream_t s, Timer* t) {
   timer_begin(t, "rstar", s);
-  k_rstar<<<b.H, BIG, 0, s>>>(b, w, kp.sync_heads);
+  const cudaError_t e = launch_kernel(k_rstar, dim3(b.H), BIG, 0, 1, true, s, b, w, kp.sync_heads);
   timer_end(t, s);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_select(const Bank& b, const Ws& w, int eviction, cudaStream_t s, Timer* t) {
+  // blocks per head: as many as fit beside each other (two blocks of 1,024 threads per SM),
+  // but no fewer than 1,024 slots each
+  int C = 8;
+  while (C > 1 && ((int64_t)b.H * C > 2 * (int64_t)sm_count() || b.M_max < 1024 * C)) C >>= 1;
+  const int cap = ((b.M_max + C - 1) / C + 31) & ~31;
   timer_begin(t, "select", s);
-  k_select<<<b.H, BIG, sel_smem_bytes(b.M_max), s>>>(b, w, eviction);
+  const cudaError_t e = launch_kernel(k_select, dim3(b.H * C), BIG, sel_smem_bytes(cap), C, true, s, b, w, eviction, cap);
   timer_end(t, s);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_commit(const Bank& b, const Ws& w, const void* Vc, int N, const int32_t* src_map, cudaStream_t s,
@@ -1153,9 +1237,9 @@ cudaError_t launch_commit(const Bank& b, const Ws& w, const void* Vc, int N, con
   const int want = n_sm > 0 ? std::max(2, (16 * n_sm + b.H - 1) / b.H) : full;
   dim3 grid(std::min(full, want), b.H);
   timer_begin(t, "commit", s);
-  k_commit<<<grid, 256, 0, s>>>(b, w, (const char*)Vc, N, b.bf16 ? 2 : 4, src_map);
+  const cudaError_t e = launch_kernel(k_commit, grid, 256, 0, 1, false, s, b, w, (const char*)Vc, N, b.bf16 ? 2 : 4, src_map);
   timer_end(t, s);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_seq_gather(const Bank& b, const Ws& w, const void* Kc, const void* Vc, int N, void* Kseq,

@@ -95,7 +95,14 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
   int nrows = 0, c0 = 0, c1 = 0;
   if (mode == PM_SCORE) { nrows = hd.empty ? 0 : N;                 c1 = hd.m_old; }
   if (mode == PM_CROSS) { nrows = hd.empty ? 0 : hd.m_old;          c1 = rmax; }
-  if (mode == PM_PROJECT) { nrows = hd.empty ? 0 : hd.m_old;        c0 = (hd.r / SNAP) * SNAP; c1 = hd.r; }
+  if (mode == PM_PROJECT) {
+    nrows = hd.empty ? 0 : hd.m_old;
+    c0 = (hd.r / SNAP) * SNAP;
+    c1 = hd.r;
+    // the whole tested range: the crossing pass's final sums are in the slot after the last
+    // full snapshot, no column is left to add
+    if (hd.r == rmax) c0 = c1 = (hd.r + SNAP - 1) / SNAP * SNAP;
+  }
   if (mode == PM_SUB) { nrows = hd.empty ? 0 : hd.m_old - hd.e;     c1 = hd.e; }
   if (mode == PM_NEWBASE) { nrows = hd.r;                           c1 = hd.m_new; }
   const int row0 = blockIdx.x * RT;
@@ -138,7 +145,8 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
             if (cross == INT_MAX && S >= thr) cross = t0 + c + 1;
           });
           static_assert(simt::CT == SNAP, "a snapshot at every tile end");
-          if (active && nc == simt::CT) snap_row[(t0 + simt::CT) / SNAP] = S;
+          // (a partial last tile's is the sum over all columns)
+          if (active) snap_row[(t0 + simt::CT) / SNAP] = S;
         } else if (mode == PM_NEWBASE) {
           simt::for_columns(nc, w, [&](int c, float x) { S = __fadd_rn(S, t0 + c == self ? 0.f : x); });
         } else {

@@ -816,8 +816,7 @@ __device__ __forceinline__ int cl_read(const int* p, int z) {
 // counts (ascending slots, as one block over all slots gives).  Bound by latency: passes over
 // the slots and barriers, so the slots are spread as far as the heads leave SMs free.
 // Measured (us, one block per head -> cluster): 12 heads x 9,360 slots 33 -> 25, x 32,760
-// 134 -> 44 (clusters of 8); 160 heads keep one block each (72 -> 82 with the cluster's
-// barriers around it, against 491 us of the pass that follows).
+// 134 -> 44 (clusters of 8); 160 heads x 2,340 to 18,720 slots 72 -> 69 (clusters of 2).
 __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int cap_max) {
   extern __shared__ uint32_t s_stage[];   // [cap] sort keys, then [(cap + 31) / 32] mandatory bits
   __shared__ int s_hist[2][256];          // this block's histogram of even and odd passes
@@ -1214,10 +1213,10 @@ cudaError_t launch_rstar(const Bank& b, const Ws& w, const KParams& kp, cudaStre
 }
 
 cudaError_t launch_select(const Bank& b, const Ws& w, int eviction, cudaStream_t s, Timer* t) {
-  // blocks per head: as many as fit beside each other (two blocks of 1,024 threads per SM),
-  // but no fewer than 1,024 slots each
+  // blocks per head: up to two rounds of the two blocks of 1,024 threads that an SM holds, and
+  // no fewer than 1,024 slots each
   int C = 8;
-  while (C > 1 && ((int64_t)b.H * C > 2 * (int64_t)sm_count() || b.M_max < 1024 * C)) C >>= 1;
+  while (C > 1 && ((int64_t)b.H * C > 4 * (int64_t)sm_count() || b.M_max < 1024 * C)) C >>= 1;
   const int cap = ((b.M_max + C - 1) / C + 31) & ~31;
   timer_begin(t, "select", s);
   const cudaError_t e = launch_kernel(k_select, dim3(b.H * C), BIG, sel_smem_bytes(cap), C, true, s, b, w, eviction, cap);

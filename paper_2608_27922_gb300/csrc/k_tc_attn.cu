@@ -133,6 +133,15 @@ constexpr int SPLIT_UNIT = 16;
 constexpr int SPLIT_CTAS = 152;              // most shares (the SMs of the GPU): sizes the scratch
 constexpr int PART_FLOATS = BQ * 128 + BQ;   // O [32 column groups][128 rows] float4, then lse [128]
 
+// Estimated time of equal shares, in key tiles of one unit (0.775 us each on an SM that has
+// work, measured with 12 full heads): `per` units a CTA of nt tiles on average, one more
+// segment (each C0 tiles of fixed cost), and the store and merge of the parts.
+constexpr float C0 = 6.f, MERGE = 16.f;
+__host__ __device__ __forceinline__ float est_shares(float per, float nt) {
+  const float t = per * nt;
+  return (t > SPLIT_MIN ? t : (float)SPLIT_MIN) + (per + 1.f) * C0 + MERGE;
+}
+
 // Key tiles of a head's units.
 __device__ __forceinline__ int unit_tiles(const AttnJob& j, int h) {
   const int m = min(max(j.b.occ[h], 0), j.b.M_max);
@@ -168,11 +177,12 @@ struct TileCursor {
       if (h >= j.b.H) return 0;   // past the end
     }
   }
-  // Share boundary t, 0 <= t <= total, moved to the start of its unit if that is not cut.
-  __device__ __forceinline__ int snap(const AttnJob& j, int nqt, int t, int total) {
+  // Share boundary t, 0 <= t <= total, moved to the start of its unit if that has fewer than
+  // `cut` tiles.
+  __device__ __forceinline__ int snap(const AttnJob& j, int nqt, int t, int total, int cut) {
     if (t >= total) return total;
     const int su = seek(j, nqt, t);
-    return su < SPLIT_UNIT ? t - (t - base) % su : t;
+    return su < cut ? t - (t - base) % su : t;
   }
 };
 
@@ -222,14 +232,25 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (SPLIT) {
     pdl_trigger();   // the merge's blocks start as SMs free up, and wait there
     if (warp == 0) {
-      int mine = 0;
-      for (int hh = lane; hh < j.b.H; hh += 32) mine += unit_tiles(j, hh);
+      int mine = 0, longest = 0;
+      for (int hh = lane; hh < j.b.H; hh += 32) {
+        const int n = unit_tiles(j, hh);
+        mine += n;
+        longest = max(longest, n);
+      }
       total = __reduce_add_sync(0xffffffffu, mine) * nqt;
-      shares = min((int)gridDim.x, max(j.b.H * nqt, total / SPLIT_MIN));
+      longest = __reduce_max_sync(0xffffffffu, longest);
+      const int units = j.b.H * nqt;
+      shares = min((int)gridDim.x, max(units, total / SPLIT_MIN));
+      // the host chose from the budgets; where the banks hold less, whole units may be shorter
+      // after all (at most one per CTA: no second wave to fill)
+      const bool whole = units <= (int)gridDim.x &&
+                         (float)longest + C0 <= est_shares((float)units / gridDim.x, (float)total / units);
+      const int cut = whole ? INT_MAX : SPLIT_UNIT;
       if ((int)blockIdx.x < shares) {
-        lo = cur.snap(j, nqt, (int)((int64_t)blockIdx.x * total / shares), total);
+        lo = cur.snap(j, nqt, (int)((int64_t)blockIdx.x * total / shares), total, cut);
         TileCursor end = cur;
-        hi = end.snap(j, nqt, (int)((int64_t)(blockIdx.x + 1) * total / shares), total);
+        hi = end.snap(j, nqt, (int)((int64_t)(blockIdx.x + 1) * total / shares), total, cut);
       }
       if (lane == 0) j.meta[blockIdx.x] = make_int4(0, 0, 0, 0);
     }
@@ -593,7 +614,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // added in that order with weights 2^(lse - max lse).  Thread = (row, four columns).  A row
 // whose weight is not finite in some part is 0, as a row whose sum is not is in one piece.
 constexpr int MG_ROWS = 8;
-constexpr int MG_UNROLL = 4;
+constexpr int MG_UNROLL = 8;
 
 __global__ void __launch_bounds__(MG_ROWS * 32) tc_attend_merge(AttnJob j) {
   pdl_wait();
@@ -603,12 +624,19 @@ __global__ void __launch_bounds__(MG_ROWS * 32) tc_attend_merge(AttnJob j) {
   const int n = u.z - i + 1;                   // parts
   const int row = blockIdx.y * MG_ROWS + threadIdx.x % MG_ROWS, c4 = threadIdx.x / MG_ROWS;
   const int qrow = u.y * BQ + row;
-  if (qrow >= j.Nq) return;
   auto slot = [&](int k) { return j.part + (int64_t)(k == 0 ? 2 * i + 1 : 2 * (i + k)) * PART_FLOATS; };
+  // the parts' lse of these rows, all loads at once (one by one, 31 parts of a lone unit were
+  // 31 trips to L2)
+  __shared__ float s_lse[SPLIT_CTAS][MG_ROWS];
+  for (int e = threadIdx.x; e < n * MG_ROWS; e += MG_ROWS * 32)
+    s_lse[e / MG_ROWS][e % MG_ROWS] = slot(e / MG_ROWS)[BQ * 128 + blockIdx.y * MG_ROWS + e % MG_ROWS];
+  __syncthreads();
+  if (qrow >= j.Nq) return;
+  const int lr = threadIdx.x % MG_ROWS;
   float mx = -INFINITY;
   bool bad = false;
   for (int k = 0; k < n; ++k) {
-    const float l = slot(k)[BQ * 128 + row];
+    const float l = s_lse[k][lr];
     bad = bad || isnan(l) || l == INFINITY;
     mx = fmaxf(mx, l);
   }
@@ -621,9 +649,8 @@ __global__ void __launch_bounds__(MG_ROWS * 32) tc_attend_merge(AttnJob j) {
 #pragma unroll
       for (int q = 0; q < MG_UNROLL; ++q)
         if (k0 + q < n) {
-          const float* p = slot(k0 + q);
-          x[q] = reinterpret_cast<const float4*>(p)[c4 * BQ + row];
-          w[q] = exp2f(p[BQ * 128 + row] - mx);
+          x[q] = reinterpret_cast<const float4*>(slot(k0 + q))[c4 * BQ + row];
+          w[q] = exp2f(s_lse[k0 + q][lr] - mx);
         }
 #pragma unroll
       for (int q = 0; q < MG_UNROLL; ++q)
@@ -981,17 +1008,15 @@ cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, 
   const int64_t units = (int64_t)((Nq + BQ - 1) / BQ) * b.H;
   const int64_t ctas2 = (int64_t)((Nq + 2 * BQ - 1) / (2 * BQ)) * b.H;
   AttnJob job{b, w.L, Nq, W, (__nv_bfloat16*)O, 1.4426950408889634f / sqrtf(128.0f), nullptr, nullptr};
-  // Schedule: the shortest of three estimates, in key tiles of one unit (0.775 us each on an
-  // SM that has work, measured with 12 full heads) from the budgets, which the host knows
-  // (occupancies it does not).  C0 tiles are a CTA's or a segment's fixed cost.
+  // Schedule: the shortest of three estimates, in key tiles of one unit, from the budgets,
+  // which the host knows (occupancies it does not).
   //   whole units, one CTA each:   every wave lasts a unit; a lone wave its longest unit
-  //   equal shares:                all SMs busy to the end, one more segment and the merge
+  //   equal shares:                all SMs busy to the end (est_shares)
   //   two query tiles per CTA:     0.92 of the time per unit (K and V cross from L2 once for
   //                                both), waves of two units
   // Both sides of the lines, us (whole units | shares | two tiles), 9,360 + 4,680 keys: 12
   // heads x 4,680 queries 249 | 264 | -; x 1,560 170 | 112 | -; x 256 95 | 37 | -; 16 heads x
-  // 4,680 - | 341 | 315; 17 heads - | 385 | 460.
-  constexpr float C0 = 6.f, MERGE = 10.f;
+  // 4,680 - | 341 | 315; 17 heads - | 406 | 460; 7 heads x 1,846 queries x 5,903 keys 40 | 47 | -.
   const int wt = (W + BK - 1) / BK;
   const float nt_max = (float)((b.M_max + BK - 1) / BK + wt);
   const float nt = (float)w.n_mtiles / b.H + wt;
@@ -1001,7 +1026,7 @@ cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, 
   const int n_cta = std::min(n_sm, SPLIT_CTAS);
   const float per = (float)units / n_cta;
   const float t_share = w.attn_part && nt_max >= SPLIT_UNIT && units < 1024
-                            ? std::max((float)SPLIT_MIN, per * nt) + (per + 1) * C0 + MERGE
+                            ? est_shares(per, nt)
                             : INFINITY;
   timer_begin(t, "attend_tc", s);
   cudaError_t e = cudaSuccess;

@@ -476,7 +476,7 @@ dkv_status_t dkv_bank_evict(dkv_bank_t bank, void* stream) {
   return cuda_status(e);
 }
 
-dkv_status_t dkv_bank_commit(dkv_bank_t bank, void* stream) {
+static dkv_status_t commit_impl(dkv_bank_t bank, bool after, void* stream) {
   NvtxRange nvtx_range("dkv_bank_commit");
   if (!bank) return DKV_ERR_ARG;
   if (bank->state != 2) return DKV_ERR_STATE;
@@ -487,7 +487,7 @@ dkv_status_t dkv_bank_commit(dkv_bank_t bank, void* stream) {
   const KParams& kp = bank->kp;
   bank->last = s;
   bank->state = 0;
-  cudaError_t e = launch_commit(b, w, bank->Vc, bank->N, bank->src_map, s, t);
+  cudaError_t e = launch_commit(b, w, bank->Vc, bank->N, bank->src_map, after, s, t);
   if (t->on && !t->attend_only) {
     // every launch timed: the two passes one after the other on `stream`, so that each
     // launch's time is its own
@@ -507,11 +507,13 @@ dkv_status_t dkv_bank_commit(dkv_bank_t bank, void* stream) {
   return cuda_status(e);
 }
 
+dkv_status_t dkv_bank_commit(dkv_bank_t bank, void* stream) { return commit_impl(bank, false, stream); }
+
 dkv_status_t dkv_bank_compress(dkv_bank_t bank, void* stream) {
   if (!bank) return DKV_ERR_ARG;
   if (bank->state != 1) return DKV_ERR_STATE;
   const dkv_status_t st = dkv_bank_evict(bank, stream);
-  return st != DKV_OK ? st : dkv_bank_commit(bank, stream);
+  return st != DKV_OK ? st : commit_impl(bank, true, stream);
 }
 
 // ---- sequential admission (within-block competition)

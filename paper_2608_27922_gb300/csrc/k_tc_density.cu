@@ -1494,7 +1494,10 @@ cudaError_t launch_tc(const Bank& b, const Ws& w, const KParams& kp, const void*
   }
   const int n_sm = sm_count();
   if constexpr (MODE == TM_CROSS) {
-    if (DKV_CROSS_DUAL && !kv && n_sm > 0) {   // the persistent two-row-tile form
+    // the persistent two-row-tile form, unless even single row tiles leave SMs idle: then one
+    // row tile per CTA, with the same sums (us, pairs | single: 24 pairs x 2,000 columns 28 |
+    // 23, 12 x 1,000 17 | 15; 148 x 4,680 52 | 54)
+    if (DKV_CROSS_DUAL && !kv && n_sm > 0 && 2 * w.n_mpairs > n_sm) {
       TcJob job{b, w, kp, 0, 0};
       timer_begin(t, name, s);
       auto* k = kp.p == 1 ? tc_cross_dual<1> : kp.p == 4 ? tc_cross_dual<4> : tc_cross_dual<2>;

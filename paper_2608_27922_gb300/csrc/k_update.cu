@@ -324,6 +324,76 @@ __device__ __forceinline__ void rope_lane(float* x, int pl, int e0, int d, int l
   }
 }
 
+// The candidates' norms for bf16 keys of 128 elements (16-byte rows and bases): a warp takes
+// 8 rows, each half of it a row at a time with one 16-byte load per lane and row, all loads
+// before the reductions; half the load and store instructions per byte of row_norms_body.
+// The sum is formed as there (four elements a chain, then the tree over the 32 chains, whose
+// last step is the lane's own pair), so both give the same bits.  160 heads x 4,680 rows: 87.5
+// -> 63.4 us (240 MB, 3.8 TB/s).
+constexpr int NW_ROWS = 8;
+
+__device__ __forceinline__ void sq_pairs(const __nv_bfloat16* p, float& a, float& b) {
+  const uint4 u = *reinterpret_cast<const uint4*>(p);
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+  float x[8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    x[2 * k] = __uint_as_float(w[k] << 16);
+    x[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+  }
+  a = fmaf(x[3], x[3], fmaf(x[2], x[2], fmaf(x[1], x[1], x[0] * x[0])));
+  b = fmaf(x[7], x[7], fmaf(x[6], x[6], fmaf(x[5], x[5], x[4] * x[4])));
+}
+
+__device__ __forceinline__ void cand_norms_wide(const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
+                                                int N, float* __restrict__ out, int64_t out_hs,
+                                                __nv_bfloat16* __restrict__ ext, int64_t ext_hs, float goff) {
+  const int h = blockIdx.y;
+  const int row0 = (blockIdx.x * (blockDim.x / 32) + warp_id()) * NW_ROWS;
+  if (row0 >= N) return;
+  const int half = lane_id() >> 4, l = lane_id() & 15;
+  float a[NW_ROWS / 2], b[NW_ROWS / 2];
+#pragma unroll
+  for (int q = 0; q < NW_ROWS / 2; ++q) {
+    const int row = row0 + 2 * q + half;
+    a[q] = b[q] = 0.f;
+    if (row < N) {
+      const int64_t off = ((int64_t)h * N + row) * 128 + l * 8;
+      sq_pairs(K + off, a[q], b[q]);
+      if (V) {   // [K; V] descriptor
+        float c, d;
+        sq_pairs(V + off, c, d);
+        a[q] += c;
+        b[q] += d;
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NW_ROWS / 2; ++q) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      a[q] += __shfl_xor_sync(0xffffffffu, a[q], o);
+      b[q] += __shfl_xor_sync(0xffffffffu, b[q], o);
+    }
+    const float n2 = a[q] + b[q];
+    const int row = row0 + 2 * q + half;
+    if (row >= N) continue;
+    if (l == 0) out[(int64_t)h * out_hs + row] = n2;
+    __nv_bfloat16 g[3], hh[3];
+    split3(-(0.5f * n2 + goff), g[0], g[1], g[2]);
+    split3(-(0.5f * n2), hh[0], hh[1], hh[2]);
+    // row form [g, g, g, 1, 1, 1, 0 ..], column form [1, 1, 1, h, h, h, 0 ..]: two values a lane
+    const __nv_bfloat16 one = __float2bfloat16_rn(1.0f), zero = __float2bfloat16_rn(0.0f);
+    __nv_bfloat162 v(zero, zero);
+    if (l == 0) v = __nv_bfloat162(g[0], g[1]);
+    else if (l == 1) v = __nv_bfloat162(g[2], one);
+    else if (l == 2 || l == 8) v = __nv_bfloat162(one, one);
+    else if (l == 9) v = __nv_bfloat162(one, hh[0]);
+    else if (l == 10) v = __nv_bfloat162(hh[1], hh[2]);
+    *reinterpret_cast<__nv_bfloat162*>(ext + (int64_t)h * ext_hs + (int64_t)row * 32 + 2 * l) = v;
+  }
+}
+
 template <typename T>
 __global__ void k_row_norms(const T* __restrict__ K, const T* __restrict__ V, int64_t head_stride, int rows_cap,
                             const int32_t* count, int count_is_occ, int N, float* __restrict__ out, int64_t out_hs,
@@ -350,6 +420,11 @@ __global__ void k_cand_prepare(Bank b, Ws w, const T* __restrict__ Kc, const T* 
          i += nthr)
       w.hist[i] = 0;
   }
+  if constexpr (sizeof(T) == 2)
+    if (b.d == 128) {
+      cand_norms_wide(Kc, Vc, N, w.cnorm, b.n_max, (__nv_bfloat16*)w.cext, (int64_t)b.n_max * 32, goff);
+      return;
+    }
   row_norms_body<T>(Kc, Vc, (int64_t)N * b.d, N, nullptr, 0, N, w.cnorm, b.n_max, b.d, (__nv_bfloat16*)w.cext,
                     (int64_t)b.n_max * 32, goff);
 }
@@ -810,13 +885,14 @@ __device__ __forceinline__ int cl_read(const int* p, int z) {
   return x;
 }
 
-// One cluster of 1 to 8 blocks per head, each with an equal run of the head's slots: block
+// One block per head (CL = false) or one cluster of 2 to 8 per head, each with an equal run of the head's slots: block
 // counts and radix histograms are added over the cluster through its shared memory, every
 // block finds the same threshold, and writes its part of the lists behind the lower ranks'
 // counts (ascending slots, as one block over all slots gives).  Bound by latency: passes over
 // the slots and barriers, so the slots are spread as far as the heads leave SMs free.
 // Measured (us, one block per head -> cluster): 12 heads x 9,360 slots 33 -> 25, x 32,760
 // 134 -> 44 (clusters of 8); 160 heads x 2,340 to 18,720 slots 72 -> 69 (clusters of 2).
+template <bool CL>
 __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int cap_max) {
   extern __shared__ uint32_t s_stage[];   // [cap] sort keys, then [(cap + 31) / 32] mandatory bits
   __shared__ int s_hist[2][256];          // this block's histogram of even and odd passes
@@ -827,7 +903,11 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int 
   __shared__ unsigned long long s_tprefix;
   pdl_wait();
   pdl_trigger();
-  const int C = cl_size(), rank = cl_rank();
+  const int C = CL ? cl_size() : 1, rank = CL ? cl_rank() : 0;
+  auto all_sync = [&]() {
+    if (CL) cl_sync();
+    else __syncthreads();
+  };
   const int h = blockIdx.x / C;
   const DevHead hd = w.hd[h];
   const int64_t bh = (int64_t)h * b.M_max;
@@ -842,6 +922,7 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int 
   if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   auto cluster_cnt = [&](int which, int ranks) {   // sum over the first `ranks` blocks
+    if (!CL) return ranks ? s_cnt[which] : 0;
     int x = 0;
     for (int z = 0; z < ranks; ++z) x += cl_read(&s_cnt[which], z);
     return x;
@@ -870,7 +951,7 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int 
     atomicAdd(&s_cnt[0], nm);
     atomicAdd(&s_cnt[1], npre);
   }
-  cl_sync();
+  all_sync();
   int n_mand = cluster_cnt(0, C);
   if (rank == 0 && threadIdx.x == 0) {
     w.hd[h].n_mand = n_mand;
@@ -879,7 +960,7 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int 
   if (e == 0 || n_mand > e) {   // (the whole cluster)
     // n_mand > e: the prefix was feasible, so this cannot happen
     if (e > 0 && rank == 0 && threadIdx.x == 0) dev_fail(w.L, DEV_INCONSISTENT, 2000 + h);
-    cl_sync();                  // no block ends while another reads its counts
+    if (CL) cl_sync();          // no block ends while another reads its counts
     return;
   }
   // Eviction policy: threshold crossers first (default and mandatory + source), or none
@@ -911,10 +992,11 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int 
       const bool v = i < hi && digit(i, &d);
       hist_add(hist, v, d);
     }
-    cl_sync();
+    all_sync();
     if (threadIdx.x < 256) {
-      int x = 0;
-      for (int z = 0; z < C; ++z) x += cl_read(&hist[threadIdx.x], z);
+      int x = CL ? 0 : hist[threadIdx.x];
+      if (CL)
+        for (int z = 0; z < C; ++z) x += cl_read(&hist[threadIdx.x], z);
       s_sum[threadIdx.x] = x;
     }
     __syncthreads();
@@ -960,7 +1042,7 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int 
       if (!is_mand(i) && key_of(i) == T) ++n_eq_local;
   n_eq_local = __reduce_add_sync(0xffffffffu, n_eq_local);
   if (lane_id() == 0 && n_eq_local) atomicAdd(&s_cnt[2], n_eq_local);
-  cl_sync();
+  all_sync();
   const unsigned n_eq = (unsigned)cluster_cnt(2, C);
   unsigned long long tprefix = 0, tmask = 0;
   const bool need_tie = k > 0 && n_eq > take_eq;   // (the whole cluster)
@@ -994,13 +1076,13 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int 
     return key > T || (key == T && (!need_tie || prov_of(i) <= tprefix));
   };
   int mine = 0;
-  if (C > 1) {   // evicted slots of each block, for the offsets of the later ones
+  if (CL) {   // evicted slots of each block, for the offsets of the later ones
     for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) mine += is_evicted(i);
     mine = __reduce_add_sync(0xffffffffu, mine);
     if (lane_id() == 0 && mine) atomicAdd(&s_cnt[3], mine);
     cl_sync();
   }
-  int n_ev = C > 1 ? cluster_cnt(3, rank) : 0;
+  int n_ev = CL ? cluster_cnt(3, rank) : 0;
   int n_sv = lo - n_ev;
   for (int base = lo; base < hi; base += blockDim.x) {
     const int i = base + threadIdx.x;
@@ -1014,7 +1096,7 @@ __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int 
     n_sv += min((int)blockDim.x, hi - base) - tot;
   }
   if (rank == C - 1 && threadIdx.x == 0 && n_ev != e) dev_fail(w.L, DEV_INCONSISTENT, 3000 + h);
-  if (C > 1) cl_sync();   // no block ends while another reads its counts
+  if (CL) cl_sync();   // no block ends while another reads its counts
 }
 
 // 1 / b of every occupied bank slot (after an import; the update keeps it in step).
@@ -1138,7 +1220,8 @@ static float ext_goff(const KParams& kp) { return kp.eps * 0.5f / kp.inv_s2; }  
 cudaError_t launch_cand_norms(const Bank& b, const Ws& w, const void* Kc, const void* Vc, int N, int64_t step,
                               const KParams& kp, const RopeArgs* rope, cudaStream_t s, Timer* t) {
   if (!w.vperm) Vc = nullptr;   // values enter the norms with the [K; V] descriptor only
-  dim3 grid((N + 8 * NR_ROWS - 1) / (8 * NR_ROWS) + 1, b.H);   // + the prepare block
+  const int per = 8 * (b.bf16 && b.d == 128 ? NW_ROWS : NR_ROWS);   // rows per CTA
+  dim3 grid((N + per - 1) / per + 1, b.H);   // + the prepare block
   const float goff = ext_goff(kp);
   cudaError_t e;
   timer_begin(t, "cand_norms", s);
@@ -1213,19 +1296,22 @@ cudaError_t launch_rstar(const Bank& b, const Ws& w, const KParams& kp, cudaStre
 }
 
 cudaError_t launch_select(const Bank& b, const Ws& w, int eviction, cudaStream_t s, Timer* t) {
-  // blocks per head: up to two rounds of the two blocks of 1,024 threads that an SM holds, and
-  // no fewer than 1,024 slots each
-  int C = 8;
-  while (C > 1 && ((int64_t)b.H * C > 4 * (int64_t)sm_count() || b.M_max < 1024 * C)) C >>= 1;
+  // blocks per head: up to two rounds of the two blocks of 1,024 threads that an SM holds, in
+  // banks of 8,192 slots or more and no fewer than 2,048 slots each (below, the cluster's
+  // barriers and remote reads cost more than the passes: 3,000 slots 15 us in one block, 19 in
+  // two)
+  int C = b.M_max < 8192 ? 1 : 8;
+  while (C > 1 && ((int64_t)b.H * C > 4 * (int64_t)sm_count() || b.M_max < 2048 * C)) C >>= 1;
   const int cap = ((b.M_max + C - 1) / C + 31) & ~31;
   timer_begin(t, "select", s);
-  const cudaError_t e = launch_kernel(k_select, dim3(b.H * C), BIG, sel_smem_bytes(cap), C, true, s, b, w, eviction, cap);
+  const cudaError_t e = launch_kernel(C > 1 ? k_select<true> : k_select<false>, dim3(b.H * C), BIG,
+                                      sel_smem_bytes(cap), C, true, s, b, w, eviction, cap);
   timer_end(t, s);
   return e;
 }
 
-cudaError_t launch_commit(const Bank& b, const Ws& w, const void* Vc, int N, const int32_t* src_map, cudaStream_t s,
-                          Timer* t) {
+cudaError_t launch_commit(const Bank& b, const Ws& w, const void* Vc, int N, const int32_t* src_map, bool after,
+                          cudaStream_t s, Timer* t) {
   // rows: ns survivors + r admitted = m_new <= M_max per head, grid-stride over them.  A
   // head's CTAs cover its largest possible row range in one pass only when the heads are
   // few: with many heads, whose layers mostly admit nothing, each head gets a few CTAs
@@ -1236,7 +1322,7 @@ cudaError_t launch_commit(const Bank& b, const Ws& w, const void* Vc, int N, con
   const int want = n_sm > 0 ? std::max(2, (16 * n_sm + b.H - 1) / b.H) : full;
   dim3 grid(std::min(full, want), b.H);
   timer_begin(t, "commit", s);
-  const cudaError_t e = launch_kernel(k_commit, grid, 256, 0, 1, false, s, b, w, (const char*)Vc, N, b.bf16 ? 2 : 4, src_map);
+  const cudaError_t e = launch_kernel(k_commit, grid, 256, 0, 1, after, s, b, w, (const char*)Vc, N, b.bf16 ? 2 : 4, src_map);
   timer_end(t, s);
   return e;
 }
@@ -1256,7 +1342,11 @@ cudaError_t update_set_smem_limits() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_sort_rank<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * RUN * 8);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sel_smem_bytes(SEL_STAGE));
+    e = cudaFuncSetAttribute(k_select<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sel_smem_bytes(SEL_STAGE));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sel_smem_bytes(SEL_STAGE));
   return e;
 }
 

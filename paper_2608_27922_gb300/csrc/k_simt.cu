@@ -9,10 +9,10 @@
 // same order in the crossing pass and in the projection pass that later resumes them from a
 // snapshot, and sums do not depend on the tile size.
 // Measured at 2,070 MHz (us, two threads per row pair before -> tiled), 12 heads, bf16, d =
-// 128: scores 1,560 x 9,360 6,957 -> 1,852, crossings 9,360 x 1,560 1,934 -> 1,864, survivors
-// 7,800 x 1,560 1,590 -> 1,505, new baselines 1,560 x 9,360 4,263 -> 1,851 (24 T fp32
-// operations/s, the packed pipe 65 to 70% busy); 2 heads, fp32, d = 64, scores 256 x 512
-// 144 -> 23.
+// 128: scores 1,560 x 9,360 6,957 -> 1,784, crossings 9,360 x 1,560 1,934 -> 1,792, survivors
+// 7,800 x 1,560 1,590 -> 1,449, new baselines 1,560 x 9,360 4,263 -> 1,789 (25 T fp32
+// operations/s, the packed pipe about 70% busy); 2 heads, fp32, d = 64, scores 256 x 512
+// 144 -> 21.
 #include "dkv_internal.h"
 #include "simt_pairs.cuh"
 
@@ -231,9 +231,9 @@ cudaError_t launch_pairs(int mode, const Bank& b, const Ws& w, const KParams& kp
 // query tile in equal parts, and each block merges a share of the rows from the others'
 // shared memory.
 // Measured at 2,070 MHz (us, one thread per query before -> this): 12 heads,
-// fp32, d = 128, 1,560 queries x 6,240 keys 4,743 -> 1,387 (43 TFLOP/s); 12 heads, d = 64,
-// 4,680 x 9,360 5,576 -> 3,231; 2 heads, d = 64, 256 x 768 315 -> 22; 1 head, d = 64,
-// 139 x 7,681 2,919 -> 46.
+// fp32, d = 128, 1,560 queries x 6,240 keys 4,743 -> 1,306 (46 TFLOP/s); 12 heads, d = 64,
+// 4,680 x 9,360 5,576 -> 3,227; 2 heads, d = 64, 256 x 768 315 -> 20; 1 head, d = 64,
+// 139 x 7,681 2,919 -> 41.
 constexpr int ANT = 128;   // threads per block
 constexpr int AK = 128;    // keys per tile
 constexpr int AC = 32;     // dimensions (keys) per staged chunk of keys (values)
@@ -288,12 +288,18 @@ __global__ void __launch_bounds__(ANT, RT == 64 ? 2 : 3)
       for (int k = 0; k < 8; ++k) x[k] = 0.f;
     }
   };
-  // chunk ch of tile t: keys' dimensions [32 ch, +32) (thread = key), then values of keys
-  // [32 (ch - NK), +32) (8-element group e: key e / (D / 8))
+  // chunk ch of tile t: dimensions [32 ch, +32) of the keys, staged as the pair passes' columns,
+  // then values of keys [32 (ch - NK), +32) (8-element group e: key e / (D / 8)).  Four threads
+  // share a key's chunk with fp32 keys (1,387 -> 1,306 us at 1,560 x 6,240, d = 128); with bf16
+  // keys, half as many lines a load, one thread per key is faster (98 against 118 us at 4 heads
+  // x 300 x 2,300)
+  constexpr bool SHARED = sizeof(T) == 4;
+  auto load_key = [&](int u) { return SHARED ? u * 32 + tid / (AC / 8) : tid; };
+  auto load_dim = [&](int u) { return 8 * (SHARED ? tid % (AC / 8) : u); };
   auto fetch = [&](int t, int ch) {
     if (ch < NK) {
 #pragma unroll
-      for (int u = 0; u < AC / 8; ++u) load(t * AK + tid, ch * AC + 8 * u, kb, kw, pre[u]);
+      for (int u = 0; u < AC / 8; ++u) load(t * AK + load_key(u), ch * AC + load_dim(u), kb, kw, pre[u]);
     } else {
 #pragma unroll
       for (int u = 0; u < LV; ++u) {
@@ -312,7 +318,8 @@ __global__ void __launch_bounds__(ANT, RT == 64 ? 2 : 3)
 #pragma unroll
       for (int u = 0; u < AC / 8; ++u)
 #pragma unroll
-        for (int k = 0; k < 8; ++k) cs[(8 * u + k) * AK + tid] = pre[u][k];
+        for (int k = 0; k < 8; ++k)
+          cs[(load_dim(u) + k) * AK + simt::swz(load_key(u), load_dim(u) + k)] = pre[u][k];
     } else {
 #pragma unroll
       for (int u = 0; u < LV; ++u) {
@@ -358,27 +365,31 @@ __global__ void __launch_bounds__(ANT, RT == 64 ? 2 : 3)
       for (int c = 0; c < TC / 2; ++c) s2[i][c] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int ch = 0; ch < NK; ++ch) {
-      const float* kp = advance(t, ch) + 4 * cg;
+      const float* kc = advance(t, ch);
       const float* qp = qs + ch * AC * RT + 4 * rg;
-#pragma unroll 4
-      for (int k = 0; k < AC; ++k) {
-        float qv[TR];
-        float2 kv[TC / 2];
+#pragma unroll 1
+      for (int k4 = 0; k4 < AC; k4 += 4) {   // (one swizzle)
+        const float* kp = kc + simt::swz(4 * cg, k4);
 #pragma unroll
-        for (int i = 0; i < TR / 4; ++i) {
-          const float4 x = *reinterpret_cast<const float4*>(qp + k * RT + i * (RT / 2));
-          qv[4 * i] = x.x; qv[4 * i + 1] = x.y; qv[4 * i + 2] = x.z; qv[4 * i + 3] = x.w;
+        for (int k = k4; k < k4 + 4; ++k) {
+          float qv[TR];
+          float2 kv[TC / 2];
+#pragma unroll
+          for (int i = 0; i < TR / 4; ++i) {
+            const float4 x = *reinterpret_cast<const float4*>(qp + k * RT + i * (RT / 2));
+            qv[4 * i] = x.x; qv[4 * i + 1] = x.y; qv[4 * i + 2] = x.z; qv[4 * i + 3] = x.w;
+          }
+#pragma unroll
+          for (int c = 0; c < TC / 4; ++c) {
+            const float4 x = *reinterpret_cast<const float4*>(kp + k * AK + c * (AK / 2));
+            kv[2 * c] = make_float2(x.x, x.y);
+            kv[2 * c + 1] = make_float2(x.z, x.w);
+          }
+#pragma unroll
+          for (int i = 0; i < TR; ++i)
+#pragma unroll
+            for (int c = 0; c < TC / 2; ++c) s2[i][c] = __ffma2_rn(make_float2(qv[i], qv[i]), kv[c], s2[i][c]);
         }
-#pragma unroll
-        for (int c = 0; c < TC / 4; ++c) {
-          const float4 x = *reinterpret_cast<const float4*>(kp + k * AK + c * (AK / 2));
-          kv[2 * c] = make_float2(x.x, x.y);
-          kv[2 * c + 1] = make_float2(x.z, x.w);
-        }
-#pragma unroll
-        for (int i = 0; i < TR; ++i)
-#pragma unroll
-          for (int c = 0; c < TC / 2; ++c) s2[i][c] = __ffma2_rn(make_float2(qv[i], qv[i]), kv[c], s2[i][c]);
       }
     }
     bool raised = false;

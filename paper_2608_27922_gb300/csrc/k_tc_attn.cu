@@ -136,7 +136,7 @@ constexpr int PART_FLOATS = BQ * 128 + BQ;   // O [32 column groups][128 rows] f
 // Estimated time of equal shares, in key tiles of one unit (0.775 us each on an SM that has
 // work, measured with 12 full heads): `per` units a CTA of nt tiles on average, one more
 // segment (each C0 tiles of fixed cost), and the store and merge of the parts.
-constexpr float C0 = 6.f, MERGE = 16.f;
+constexpr float C0 = 6.f, MERGE = 23.f;
 __host__ __device__ __forceinline__ float est_shares(float per, float nt) {
   const float t = per * nt;
   return (t > SPLIT_MIN ? t : (float)SPLIT_MIN) + (per + 1.f) * C0 + MERGE;
@@ -1017,17 +1017,27 @@ cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, 
   // Both sides of the lines, us (whole units | shares | two tiles), 9,360 + 4,680 keys: 12
   // heads x 4,680 queries 249 | 264 | -; x 1,560 170 | 112 | -; x 256 95 | 37 | -; 16 heads x
   // 4,680 - | 341 | 315; 17 heads - | 406 | 460; 7 heads x 1,846 queries x 5,903 keys 40 | 47 | -.
+  // In each, HBM: HBM_UNITS units' tiles of keys and values take it one tile's time (6.5 TB/s).
+  // Whole units in order keep the query tiles of one head side by side, which read its keys
+  // once; shares walk all heads at once, so where those do not fit L2 every unit reads its keys
+  // from HBM (whole units | shares: 123 heads x 182 queries x 15,832 keys 212 | 301, 40 x 1,560
+  // x 14,040 326 | 507; one query tile a head: 160 x 128 x 14,040 232 | 189).
+  constexpr float HBM_UNITS = 77.f;
+  constexpr double L2_BYTES = 180e6;   // (126 MB, and some reuse beyond: 24 x 1,560 x 14,040,
+                                       //  173 MB, 242 | 206)
   const int wt = (W + BK - 1) / BK;
   const float nt_max = (float)((b.M_max + BK - 1) / BK + wt);
   const float nt = (float)w.n_mtiles / b.H + wt;
   const float waves = (float)((units + n_sm - 1) / n_sm), waves2 = (float)((ctas2 + n_sm - 1) / n_sm);
-  const float t_whole = std::max(nt_max, waves * nt) + waves * C0;
+  // heads read by a full wave of whole units, and by the last one
+  const float nqt = (float)((Nq + BQ - 1) / BQ), in_wave = n_sm / nqt, in_last = b.H - (waves - 1) * in_wave;
+  const float t_waves = (waves - 1) * nt * std::max(1.f, in_wave / HBM_UNITS) + nt * std::max(1.f, in_last / HBM_UNITS);
+  const float t_whole = std::max(nt_max, t_waves) + waves * C0;
   const float t_two = ctas2 >= 2 * (int64_t)n_sm ? waves2 * (1.84f * nt + C0) : INFINITY;
   const int n_cta = std::min(n_sm, SPLIT_CTAS);
   const float per = (float)units / n_cta;
-  const float t_share = w.attn_part && nt_max >= SPLIT_UNIT && units < 1024
-                            ? est_shares(per, nt)
-                            : INFINITY;
+  float t_share = w.attn_part && nt_max >= SPLIT_UNIT && units < 1024 ? est_shares(per, nt) : INFINITY;
+  if (2.0 * TB * b.H * nt > L2_BYTES) t_share = std::max(t_share, units * nt / HBM_UNITS + 2 * C0 + MERGE);
   timer_begin(t, "attend_tc", s);
   cudaError_t e = cudaSuccess;
   if (t_two <= std::min(t_whole, t_share)) {

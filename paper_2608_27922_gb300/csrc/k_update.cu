@@ -891,7 +891,8 @@ __device__ __forceinline__ int cl_read(const int* p, int z) {
 // counts (ascending slots, as one block over all slots gives).  Bound by latency: passes over
 // the slots and barriers, so the slots are spread as far as the heads leave SMs free.
 // Measured (us, one block per head -> cluster): 12 heads x 9,360 slots 33 -> 25, x 32,760
-// 134 -> 44 (clusters of 8); 160 heads x 2,340 to 18,720 slots 72 -> 69 (clusters of 2).
+// 134 -> 43 (clusters of 4 and 8); 160 heads x 2,340 to 18,720 slots 72 in one block each, 83
+// in clusters of 2.
 template <bool CL>
 __global__ void __launch_bounds__(BIG) k_select(Bank b, Ws w, int eviction, int cap_max) {
   extern __shared__ uint32_t s_stage[];   // [cap] sort keys, then [(cap + 31) / 32] mandatory bits
@@ -1296,12 +1297,12 @@ cudaError_t launch_rstar(const Bank& b, const Ws& w, const KParams& kp, cudaStre
 }
 
 cudaError_t launch_select(const Bank& b, const Ws& w, int eviction, cudaStream_t s, Timer* t) {
-  // blocks per head: up to two rounds of the two blocks of 1,024 threads that an SM holds, in
+  // blocks per head: as many as fit beside each other (two blocks of 1,024 threads per SM), in
   // banks of 8,192 slots or more and no fewer than 2,048 slots each (below, the cluster's
   // barriers and remote reads cost more than the passes: 3,000 slots 15 us in one block, 19 in
   // two)
   int C = b.M_max < 8192 ? 1 : 8;
-  while (C > 1 && ((int64_t)b.H * C > 4 * (int64_t)sm_count() || b.M_max < 2048 * C)) C >>= 1;
+  while (C > 1 && ((int64_t)b.H * C > 2 * (int64_t)sm_count() || b.M_max < 2048 * C)) C >>= 1;
   const int cap = ((b.M_max + C - 1) / C + 31) & ~31;
   timer_begin(t, "select", s);
   const cudaError_t e = launch_kernel(C > 1 ? k_select<true> : k_select<false>, dim3(b.H * C), BIG,

@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       longest = __reduce_max_sync(0xffffffffu, longest);
       const int units = j.b.H * nqt;
       shares = min((int)gridDim.x, max(units, total / SPLIT_MIN));
-      // the host chose from the budgets; where the banks hold less, whole units may be shorter
-      // after all (at most one per CTA: no second wave to fill)
+      // the host chose from bounds; where the banks hold less, whole units may be shorter after
+      // all (at most one per CTA: no second wave to fill)
       const bool whole = units <= (int)gridDim.x &&
                          (float)longest + C0 <= est_shares((float)units / gridDim.x, (float)total / units);
       const int cut = whole ? INT_MAX : SPLIT_UNIT;
@@ -991,8 +991,8 @@ cudaError_t tc_attn_set_smem_limits() {
 
 size_t attend_scratch_bytes() { return (size_t)SPLIT_CTAS * (2 * PART_FLOATS * sizeof(float) + sizeof(int4)); }
 
-cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw,
-                             int W, void* O, cudaStream_t s, Timer* t) {
+cudaError_t launch_attend_tc(const Bank& b, const Ws& w, int64_t bank_tiles, int bank_max, const void* Q, int Nq,
+                             const void* Kw, const void* Vw, int W, void* O, cudaStream_t s, Timer* t) {
   CUtensorMap mq, mkb, mvb, mkw, mvw;
   if (!make_map_rows(&mq, Q, Nq, b.H, BQ) || !make_map_rows(&mkb, b.k, b.M_max, b.H, BK) ||
       !make_map_rows(&mvb, b.v, b.M_max, b.H, BK))
@@ -1008,8 +1008,8 @@ cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, 
   const int64_t units = (int64_t)((Nq + BQ - 1) / BQ) * b.H;
   const int64_t ctas2 = (int64_t)((Nq + 2 * BQ - 1) / (2 * BQ)) * b.H;
   AttnJob job{b, w.L, Nq, W, (__nv_bfloat16*)O, 1.4426950408889634f / sqrtf(128.0f), nullptr, nullptr};
-  // Schedule: the shortest of three estimates, in key tiles of one unit, from the budgets,
-  // which the host knows (occupancies it does not).
+  // Schedule: the shortest of three estimates, in key tiles of one unit, from the bounds of the
+  // banks' tiles that the handle keeps.
   //   whole units, one CTA each:   every wave lasts a unit; a lone wave its longest unit
   //   equal shares:                all SMs busy to the end (est_shares)
   //   two query tiles per CTA:     0.92 of the time per unit (K and V cross from L2 once for
@@ -1026,8 +1026,8 @@ cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, 
   constexpr double L2_BYTES = 180e6;   // (126 MB, and some reuse beyond: 24 x 1,560 x 14,040,
                                        //  173 MB, 242 | 206)
   const int wt = (W + BK - 1) / BK;
-  const float nt_max = (float)((b.M_max + BK - 1) / BK + wt);
-  const float nt = (float)w.n_mtiles / b.H + wt;
+  const float nt_max = (float)(bank_max + wt);
+  const float nt = (float)bank_tiles / b.H + wt;
   const float waves = (float)((units + n_sm - 1) / n_sm), waves2 = (float)((ctas2 + n_sm - 1) / n_sm);
   // heads read by a full wave of whole units, and by the last one
   const float nqt = (float)((Nq + BQ - 1) / BQ), in_wave = n_sm / nqt, in_last = b.H - (waves - 1) * in_wave;

@@ -18,7 +18,7 @@
 // (smaller score, or equal score and smaller source index): the stable ascending
 // order, without a buffer to sort in and over as many blocks as there are candidates.
 // Measured at 2,070 MHz, d = 128, bf16, 9,360 bank keys x 4,680 candidates: the
-// whole call 4,885 us before (one thread per candidate, one block sorting) -> 654.
+// whole call 4,885 us before (one thread per candidate, one block sorting) -> 531.
 #include "../../include/dkv.h"
 #include "dkv_internal.h"
 #include "simt_pairs.cuh"
@@ -35,16 +35,25 @@ static __device__ __align__(256) float g_noalloc_scores[DKV_NOALLOC_MAX_N];
 
 template <typename T, int D, int RT>
 __global__ void __launch_bounds__(simt::NT) noalloc_score(const T* Kb, const float* base, int m, const T* Kc, int N,
-                                                          KParams kp, bool vec, float* scratch) {
+                                                          KParams kp, bool vec, int cluster, float* scratch) {
   extern __shared__ __align__(16) float smem[];
-  const int row0 = blockIdx.x * RT;
+  __shared__ int4 mail[RT];
+  const int C = cluster, z = blockIdx.x % C;   // the cluster is C neighbouring blocks
+  const int row0 = blockIdx.x / C * RT;
   const int sr = simt::scan_row<RT>();
+  simt::Chain<RT> chain(mail, z, C, (m + simt::CT - 1) / simt::CT);
   float acc = 0.f;
-  simt::pair_tiles<T, D, false, RT>(Kc, nullptr, row0, N, Kb, nullptr, base, 0, m, kp, vec, smem,
-                                    [&](int, int nc, const float* w, const float* inv) {
+  int unused = 0;
+  simt::pair_tiles<T, D, false, RT>(Kc, nullptr, row0, N, Kb, nullptr, base, 0, m, kp, vec, smem, z, C,
+                                    [&](int t0, int nc, const float* w, const float* inv) {
+                                      const int t = t0 / simt::CT;
+                                      // (a hand-over that never came shows as NaN scores)
+                                      if (!chain.take(sr, t, acc, unused)) acc = __int_as_float(0x7fffffff);
                                       simt::for_columns(nc, w, [&](int c, float x) { acc = __fmaf_rn(x, inv[c], acc); });
+                                      chain.give(sr, t, acc, unused);
                                     });
-  if (sr >= 0 && row0 + sr < N) scratch[row0 + sr] = __fdiv_rn(acc, (float)m);
+  chain.finish();
+  if (chain.last() && sr >= 0 && row0 + sr < N) scratch[row0 + sr] = __fdiv_rn(acc, (float)m);
 }
 
 // Block b places candidates [32 b, 32 b + 32): thread (i, g) = (t % 32, t / 32) counts, for
@@ -109,20 +118,20 @@ __global__ void __launch_bounds__(32 * ORD_GROUPS) noalloc_order(const float* sc
 
 template <typename T, int D, int RT>
 cudaError_t launch_score(const void* Kb, const float* base, int m, const void* Kc, int N, const KParams& kp,
-                         float* scratch, cudaStream_t s) {
+                         int C, float* scratch, cudaStream_t s) {
   // this entry point asks no alignment of its key arrays beyond the element's
   const bool vec = ((reinterpret_cast<uintptr_t>(Kb) | reinterpret_cast<uintptr_t>(Kc)) & 15u) == 0;
-  noalloc_score<T, D, RT><<<(N + RT - 1) / RT, simt::NT, simt::Lay<D, false, RT>::SMEM, s>>>(
-      static_cast<const T*>(Kb), base, m, static_cast<const T*>(Kc), N, kp, vec, scratch);
-  return cudaGetLastError();
+  return launch_kernel(noalloc_score<T, D, RT>, dim3((N + RT - 1) / RT * C), simt::NT, simt::Lay<D, false, RT>::SMEM, C,
+                       false, s, static_cast<const T*>(Kb), base, m, static_cast<const T*>(Kc), N, kp, vec, C, scratch);
 }
 
 template <typename T, int D>
 cudaError_t launch_score(const void* Kb, const float* base, int m, const void* Kc, int N, const KParams& kp,
                          float* scratch, cudaStream_t s) {
-  return simt::pick_rows(1, N, sm_count(), false) == 32
-             ? launch_score<T, D, 32>(Kb, base, m, Kc, N, kp, scratch, s)
-             : launch_score<T, D, 16>(Kb, base, m, Kc, N, kp, scratch, s);
+  const simt::Shape p = simt::pick_shape(1, N, m, D, sm_count(), true);
+  return p.rows == 64   ? launch_score<T, D, 64>(Kb, base, m, Kc, N, kp, p.cluster, scratch, s)
+         : p.rows == 32 ? launch_score<T, D, 32>(Kb, base, m, Kc, N, kp, p.cluster, scratch, s)
+                        : launch_score<T, D, 16>(Kb, base, m, Kc, N, kp, p.cluster, scratch, s);
 }
 
 // Set-up per device, with that device current: the device address of the scratch
@@ -147,12 +156,16 @@ cudaError_t setup_device(int dev, float** scratch) {
     auto opt_in = [&](auto k, size_t bytes) {
       if (err == cudaSuccess) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
+    opt_in(noalloc_score<__nv_bfloat16, 128, 64>, simt::Lay<128, false, 64>::SMEM);
     opt_in(noalloc_score<__nv_bfloat16, 128, 32>, simt::Lay<128, false, 32>::SMEM);
     opt_in(noalloc_score<__nv_bfloat16, 128, 16>, simt::Lay<128, false, 16>::SMEM);
+    opt_in(noalloc_score<__nv_bfloat16, 64, 64>, simt::Lay<64, false, 64>::SMEM);
     opt_in(noalloc_score<__nv_bfloat16, 64, 32>, simt::Lay<64, false, 32>::SMEM);
     opt_in(noalloc_score<__nv_bfloat16, 64, 16>, simt::Lay<64, false, 16>::SMEM);
+    opt_in(noalloc_score<float, 128, 64>, simt::Lay<128, false, 64>::SMEM);
     opt_in(noalloc_score<float, 128, 32>, simt::Lay<128, false, 32>::SMEM);
     opt_in(noalloc_score<float, 128, 16>, simt::Lay<128, false, 16>::SMEM);
+    opt_in(noalloc_score<float, 64, 64>, simt::Lay<64, false, 64>::SMEM);
     opt_in(noalloc_score<float, 64, 32>, simt::Lay<64, false, 32>::SMEM);
     opt_in(noalloc_score<float, 64, 16>, simt::Lay<64, false, 16>::SMEM);
     if (err != cudaSuccess) {

@@ -12,7 +12,7 @@
 // 128: scores 1,560 x 9,360 6,957 -> 1,784, crossings 9,360 x 1,560 1,934 -> 1,792, survivors
 // 7,800 x 1,560 1,590 -> 1,449, new baselines 1,560 x 9,360 4,263 -> 1,789 (25 T fp32
 // operations/s, the packed pipe about 70% busy); 2 heads, fp32, d = 64, scores 256 x 512
-// 144 -> 21.
+// 144 -> 16 (over clusters of 4 blocks, Chain in simt_pairs.cuh).
 #include "dkv_internal.h"
 #include "simt_pairs.cuh"
 
@@ -87,8 +87,10 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
   extern __shared__ __align__(16) float smem[];
   pdl_wait();
   pdl_trigger();
+  __shared__ int4 mail[RT];
   const int h = blockIdx.y;
   const int mode = j.mode;   // uniform
+  const int C = simt_cluster_size(), z = simt_cluster_rank();
   const DevHead hd = j.w.hd[h];
   const int N = layer_of(j.w, h)->N;
   const int rmax = layer_of(j.w, h)->rmax;
@@ -105,11 +107,12 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
   }
   if (mode == PM_SUB) { nrows = hd.empty ? 0 : hd.m_old - hd.e;     c1 = hd.e; }
   if (mode == PM_NEWBASE) { nrows = hd.r;                           c1 = hd.m_new; }
-  const int row0 = blockIdx.x * RT;
-  if (row0 >= nrows) return;
+  const int row0 = blockIdx.x / C * RT;
+  if (row0 >= nrows) return;   // (all of a cluster)
   const int sr = simt::scan_row<RT>();
   const int row = row0 + sr;
   const bool active = sr >= 0 && row < nrows;
+  simt::Chain<RT> chain(mail, z, C, c1 > c0 ? (c1 - c0 + simt::CT - 1) / simt::CT : 0);
   const int64_t bh = (int64_t)h * j.b.M_max;   // bank head offset (rows)
 
   // state of this thread's row
@@ -122,7 +125,7 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
       thr = __fmul_rn(j.kp.tau, j.b.base[bh + row]);
       if (S >= thr) cross = 0;
       snap_row = j.w.snap + (bh + row) * j.w.snap_stride;
-      snap_row[0] = S;
+      if (z == 0) snap_row[0] = S;
     } else if (mode == PM_PROJECT) {
       S = j.w.snap[(bh + row) * j.w.snap_stride + c0 / SNAP];
     } else if (mode == PM_SUB) {
@@ -135,8 +138,10 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
   simt::pair_tiles<T, D, KV, RT>(
       ptr<T>(j.rk, (int64_t)h * j.rk_hs), KV ? ptr<T>(j.rv, (int64_t)h * j.rk_hs) : nullptr, row0, nrows,
       ptr<T>(j.ck, (int64_t)h * j.ck_hs), KV ? ptr<T>(j.cv, (int64_t)h * j.ck_hs) : nullptr,
-      mode == PM_SCORE ? j.b.base + bh : nullptr, c0, c1, j.kp, true, smem,
+      mode == PM_SCORE ? j.b.base + bh : nullptr, c0, c1, j.kp, true, smem, z, C,
       [&](int t0, int nc, const float* w, const float* meta) {
+        const int t = (t0 - c0) / simt::CT;
+        if (!chain.take(sr, t, S, cross)) dev_fail(j.w.L, DEV_TIMEOUT, 6500 + mode);
         if (mode == PM_SCORE) {
           simt::for_columns(nc, w, [&](int c, float x) { S = __fmaf_rn(x, meta[c], S); });
         } else if (mode == PM_CROSS) {
@@ -152,8 +157,10 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
         } else {
           simt::for_columns(nc, w, [&](int c, float x) { S = __fadd_rn(S, x); });
         }
+        chain.give(sr, t, S, cross);
       });
-  if (!active) return;
+  chain.finish();
+  if (!active || !chain.last()) return;
   if ((mode == PM_SUB && (slot < 0 || slot >= hd.m_old)) || (mode == PM_NEWBASE && (self < 0 || self >= hd.M))) {
     dev_fail(j.w.L, DEV_INCONSISTENT, 6000 + mode);   // a list entry out of range: skip the write
     return;
@@ -183,38 +190,42 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
 }
 
 template <typename T, int D, bool KV, int RT>
-cudaError_t launch_tile(int max_rows, cudaStream_t s, const PairJob& j) {
+cudaError_t launch_tile(int max_rows, int C, cudaStream_t s, const PairJob& j) {
   const bool after = j.mode == PM_SCORE || j.mode == PM_CROSS;   // follows another kernel of the same call
-  return launch_kernel(simt_pairs<T, D, KV, RT>, dim3((max_rows + RT - 1) / RT, j.b.H), simt::NT,
-                       simt::Lay<D, KV, RT>::SMEM, 1, after, s, j);
+  return launch_kernel(simt_pairs<T, D, KV, RT>, dim3((max_rows + RT - 1) / RT * C, j.b.H), simt::NT,
+                       simt::Lay<D, KV, RT>::SMEM, C, after, s, j);
 }
 
 template <typename T, int D, bool KV>
-cudaError_t launch_rows(int max_rows, cudaStream_t s, const PairJob& j) {
-  switch (simt::pick_rows(j.b.H, max_rows, sm_count(), !KV)) {
+cudaError_t launch_rows(int max_rows, int max_cols, cudaStream_t s, const PairJob& j) {
+  const simt::Shape p = simt::pick_shape(j.b.H, max_rows, max_cols, KV ? 2 * D : D, sm_count(), !KV);
+  switch (p.rows) {
     case 64:
-      if constexpr (!KV) return launch_tile<T, D, KV, 64>(max_rows, s, j);
+      if constexpr (!KV) return launch_tile<T, D, KV, 64>(max_rows, p.cluster, s, j);
       [[fallthrough]];
-    case 32: return launch_tile<T, D, KV, 32>(max_rows, s, j);
-    default: return launch_tile<T, D, KV, 16>(max_rows, s, j);
+    case 32: return launch_tile<T, D, KV, 32>(max_rows, p.cluster, s, j);
+    default: return launch_tile<T, D, KV, 16>(max_rows, p.cluster, s, j);
   }
 }
 
 template <typename T, int D>
-cudaError_t launch_desc(int max_rows, cudaStream_t s, const PairJob& j) {
-  return j.rv ? launch_rows<T, D, true>(max_rows, s, j) : launch_rows<T, D, false>(max_rows, s, j);
+cudaError_t launch_desc(int max_rows, int max_cols, cudaStream_t s, const PairJob& j) {
+  return j.rv ? launch_rows<T, D, true>(max_rows, max_cols, s, j) : launch_rows<T, D, false>(max_rows, max_cols, s, j);
 }
 
 // rv / cv: the row and column values, non-null only with the [K; V] descriptor.
 cudaError_t launch_pairs(int mode, const Bank& b, const Ws& w, const KParams& kp, const void* rk, int64_t rk_hs,
                          const void* ck, int64_t ck_hs, const void* rv, const void* cv, int max_rows,
-                         cudaStream_t s, Timer* t, const char* name) {
+                         int max_cols, cudaStream_t s, Timer* t, const char* name) {
   PairJob j{mode, rk, rk_hs, ck, ck_hs, rv, cv, b, w, kp};
   if (max_rows <= 0) return cudaSuccess;
   timer_begin(t, name, s);
   cudaError_t e;
-  if (b.bf16) e = b.d == 128 ? launch_desc<__nv_bfloat16, 128>(max_rows, s, j) : launch_desc<__nv_bfloat16, 64>(max_rows, s, j);
-  else e = b.d == 128 ? launch_desc<float, 128>(max_rows, s, j) : launch_desc<float, 64>(max_rows, s, j);
+  if (b.bf16)
+    e = b.d == 128 ? launch_desc<__nv_bfloat16, 128>(max_rows, max_cols, s, j)
+                   : launch_desc<__nv_bfloat16, 64>(max_rows, max_cols, s, j);
+  else
+    e = b.d == 128 ? launch_desc<float, 128>(max_rows, max_cols, s, j) : launch_desc<float, 64>(max_rows, max_cols, s, j);
   timer_end(t, s);
   return e;
 }
@@ -527,30 +538,30 @@ cudaError_t launch_score_fp32(const Bank& b, const Ws& w, const void* Kc, const 
   // rows: candidates in source order; columns: bank keys [0, m)
   const bool kv = w.vperm != nullptr;
   return launch_pairs(PM_SCORE, b, w, kp, Kc, (int64_t)N * b.d, b.k, (int64_t)b.M_max * b.d, kv ? Vc : nullptr,
-                                kv ? b.v : nullptr, N, s, t, "score_fp32");
+                                kv ? b.v : nullptr, N, b.M_max, s, t, "score_fp32");
 }
 
 cudaError_t launch_cross_fp32(const Bank& b, const Ws& w, const KParams& kp, cudaStream_t s, Timer* t) {
   const bool kv = w.vperm != nullptr;
   return launch_pairs(PM_CROSS, b, w, kp, b.k, (int64_t)b.M_max * b.d, w.kperm, (int64_t)b.n_max * b.d,
-                                kv ? b.v : nullptr, w.vperm, b.M_max, s, t, "cross_fp32");
+                                kv ? b.v : nullptr, w.vperm, b.M_max, b.n_max, s, t, "cross_fp32");
 }
 
 cudaError_t launch_project_fp32(const Bank& b, const Ws& w, const KParams& kp, cudaStream_t s, Timer* t) {
   const bool kv = w.vperm != nullptr;
   return launch_pairs(PM_PROJECT, b, w, kp, b.k, (int64_t)b.M_max * b.d, w.kperm, (int64_t)b.n_max * b.d,
-                                  kv ? b.v : nullptr, w.vperm, b.M_max, s, t, "project_fp32");
+                                  kv ? b.v : nullptr, w.vperm, b.M_max, SNAP, s, t, "project_fp32");
 }
 
 cudaError_t launch_subtract_fp32(const Bank& b, const Ws& w, const KParams& kp, cudaStream_t s, Timer* t) {
   return launch_pairs(PM_SUB, b, w, kp, w.ksurv, (int64_t)b.M_max * b.d, w.kevict, (int64_t)b.n_max * b.d,
-                              w.vsurv, w.vevict, b.M_max, s, t, "subtract_fp32");
+                              w.vsurv, w.vevict, b.M_max, b.n_max, s, t, "subtract_fp32");
 }
 
 cudaError_t launch_newbase_fp32(const Bank& b, const Ws& w, const KParams& kp, cudaStream_t s, Timer* t) {
   const bool kv = w.vperm != nullptr;
   return launch_pairs(PM_NEWBASE, b, w, kp, w.kperm, (int64_t)b.n_max * b.d, b.k, (int64_t)b.M_max * b.d,
-                                  w.vperm, kv ? b.v : nullptr, b.n_max, s, t, "newbase_fp32");
+                                  w.vperm, kv ? b.v : nullptr, b.n_max, b.M_max, s, t, "newbase_fp32");
 }
 
 namespace {
@@ -567,7 +578,7 @@ cudaError_t launch_attend_t(const Bank& b, const void* Q, int Nq, const void* Kw
 template <typename T, int D>
 cudaError_t launch_attend_d(const Bank& b, const void* Q, int Nq, const void* Kw, const void* Vw, int W, void* O,
                             cudaStream_t s) {
-  switch (simt::pick_rows(b.H, Nq, sm_count(), true)) {
+  switch (simt::pick_shape(b.H, Nq, 1, D, sm_count(), true).rows) {   // (its key split: below)
     case 64: return launch_attend_t<T, D, 64>(b, Q, Nq, Kw, Vw, W, O, 1, s);
     case 32: return launch_attend_t<T, D, 32>(b, Q, Nq, Kw, Vw, W, O, 1, s);
     default: break;

@@ -18,9 +18,12 @@
 // chunk in registers while this one is used; four neighbouring threads load a column's chunk
 // (one thread per column touched 32 cache lines with every load) and store it transposed, in
 // 16-byte groups of columns swizzled by the dimension, so that neither side meets a bank
-// conflict (12-head update of 1,560 x 9,360: 7,109 -> 6,842 us).  The 128 columns' w of a row then go through
-// shared memory to one thread, which adds them in column order: a pass's row sums keep one
-// fixed order for any tile size.
+// conflict (12-head update of 1,560 x 9,360: 7,109 -> 6,842 us).  The 128 columns' w of a
+// row then go through shared memory to one thread, which adds them in column order: a pass's
+// row sums keep one fixed order for any tile size.
+// Few rows: a cluster of C blocks takes a block's rows, block z the column tiles z, z + C, ..,
+// and the running sums go from each tile's block to the next one's through shared memory
+// (Chain), so the order of the additions stays the same.
 #pragma once
 
 #include "dkv_device.cuh"
@@ -31,6 +34,7 @@ namespace simt {
 constexpr int NT = 128;   // threads per block
 constexpr int CT = 128;   // columns per tile
 constexpr int KC = 32;    // dimensions per staged column chunk
+constexpr double CHAIN_COST = 10.0;   // see pick_shape
 constexpr int WS = CT + 4;   // row stride of the w tile (odd in 16-byte units: no bank conflicts)
 
 template <int D, bool KV, int RT>
@@ -46,23 +50,101 @@ struct Lay {
   static constexpr int META = W + RT * WS;           // float [CT]
   static constexpr int FLOATS = META + CT;
   static constexpr size_t SMEM = (size_t)FLOATS * 4;
-  static_assert(SMEM <= 227 * 1024, "shared memory per block");
+  static_assert(SMEM + RT * 16 <= 227 * 1024, "shared memory per block (with a Chain's mailboxes)");
   static_assert((RT / TR) * CG == NT, "one thread per tile of partial sums");
 };
 
-// Rows per block for H heads of `rows` rows.  The SM with the most blocks sets the time, each
-// costing its rows (16-row blocks read more shared memory per pair: 1.3 times), and one block
-// alone on its SM leaves latencies open (1.5 times); the tallest of equals.  Both sides: 12
-// heads x 1,560 rows x 9,360 columns 1,852 us with 64 rows, 1,985 with 32; 1 head x 4,680 x
-// 9,360 654 us with 16 rows (two blocks per SM), 743 with 32 (one).
-inline int pick_rows(int64_t H, int64_t rows, int64_t n_sm, bool tall) {
-  auto cost = [&](int rt, double per) {
-    const int64_t blocks = H * ((rows + rt - 1) / rt);
-    const int64_t most = (blocks + n_sm - 1) / (n_sm > 0 ? n_sm : 1);
-    return per * rt * (double)most * (most == 1 ? 1.5 : 1.0);
-  };
-  const double c64 = tall ? cost(64, 1.0) : 1e30, c32 = cost(32, 1.05), c16 = cost(16, 1.3);
-  return c64 <= c32 && c64 <= c16 ? 64 : c32 <= c16 ? 32 : 16;
+// Hands a row's running state from the block that has added column tile t to the one that
+// adds tile t + 1 (rank (t + 1) % C of the cluster; nothing to do with C = 1).  Each scanning
+// thread sends to the same thread of that block: its two words, then the tile they are for.
+// A mailbox is free again when it is written next: that state has been through the receiver.
+// All of a block's threads construct and finish().
+template <int RT>
+struct Chain {
+  static constexpr uint64_t WAIT_NS = 2000000000ull;   // far above any legitimate wait
+  int4* mail;      // [RT] of this block: state x, y; tile
+  int z, C, tiles;
+  bool late = false;   // a hand-over did not come: the later ones are not waited for
+  __device__ __forceinline__ Chain(int4* m, int rank, int size, int ntiles) : mail(m), z(rank), C(size), tiles(ntiles) {
+    if (C == 1) return;
+    if (threadIdx.x < RT) mail[threadIdx.x].z = 0;
+    sync();
+  }
+  __device__ __forceinline__ void sync() const {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  }
+  // no block leaves while another may still write to it
+  __device__ __forceinline__ void finish() const {
+    if (C > 1) sync();
+  }
+  // this block holds the state after the last tile
+  __device__ __forceinline__ bool last() const { return z == (tiles > 0 ? (tiles - 1) % C : 0); }
+  // the state before tile t; false if it did not come in time
+  __device__ __forceinline__ bool take(int sr, int t, float& x, int& y) {
+    if (C == 1 || t == 0) return true;
+    if (late) return false;
+    const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(mail + sr));
+    uint64_t t0 = 0;
+    for (uint32_t it = 1;; ++it) {
+      int tag;
+      asm volatile("ld.acquire.cluster.shared::cta.b32 %0, [%1];" : "=r"(tag) : "r"(a + 8) : "memory");
+      if (tag == t) break;
+      if ((it & 255u) == 0u) {
+        const uint64_t now = globaltimer_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > WAIT_NS) {
+          late = true;
+          return false;
+        }
+      }
+    }
+    const volatile int4* m = mail + sr;
+    x = __int_as_float(m->x);
+    y = m->y;
+    return true;
+  }
+  __device__ __forceinline__ void give(int sr, int t, float x, int y) const {
+    if (C == 1 || t + 1 >= tiles) return;
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;"
+        : "=r"(a)
+        : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(mail + sr))), "r"((z + 1) % C));
+    asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(__float_as_int(x)), "r"(y) : "memory");
+    asm volatile("st.release.cluster.shared::cluster.b32 [%0], %1;" ::"r"(a + 8), "r"(t + 1) : "memory");
+  }
+};
+
+// Rows and cluster size for H heads of `rows` rows against `cols` columns of `dims` elements.
+// The SM with the most blocks sets the time, each costing its rows and tiles (16-row blocks
+// read more shared memory per pair: 1.3 times), and one block alone on its SM leaves latencies
+// open (1.5 times); in a cluster every block adds its start, end and hand-overs (CHAIN_COST).
+// The smallest cluster and the tallest block of equals.  Both sides, us (16 rows, one block |
+// chosen | next best): 1 head x 1,560 rows x 9,360 columns 564 | 196 (32 rows, 8 blocks) | 242;
+// x 4,680 x 9,360 660 | 531 (64, 4) | 561; 2 heads x 256 x 512, d = 64 23.9 | 16.2 (16, 4) |
+// 17.4; 8 x 128 x 4,000 218 | 77 (32, 8) | 82.  More blocks lose where rows fill the SMs: 1 x
+// 9,360 x 1,560 189 (32, 1) | 204 (32, 4); 12 x 9,360 x 1,560 1,800 (64, 1) | 1,939 (64, 2).
+struct Shape {
+  int rows, cluster;
+};
+inline Shape pick_shape(int64_t H, int64_t rows, int64_t cols, int dims, int64_t n_sm, bool tall) {
+  const int64_t tiles = cols > CT ? (cols + CT - 1) / CT : 1;
+  const double unit = dims / 128.0;   // cost of one row and tile (1: 0.19 us)
+  Shape best{16, 1};
+  double least = 1e300;
+  for (int C = 1; C <= 8 && C <= tiles; C *= 2)
+    for (int rt = tall ? 64 : 32; rt >= 16; rt /= 2) {
+      const int64_t blocks = H * ((rows + rt - 1) / rt) * C;
+      const int64_t most = (blocks + n_sm - 1) / (n_sm > 0 ? n_sm : 1);
+      const double per = rt == 64 ? 1.0 : rt == 32 ? 1.05 : 1.3;
+      double c = unit * per * rt * (double)most * (double)((tiles + C - 1) / C) * (most == 1 ? 1.5 : 1.0);
+      if (C > 1) c += CHAIN_COST * (double)most;
+      if (c < least) {
+        least = c;
+        best = Shape{rt, C};
+      }
+    }
+  return best;
 }
 
 // Place of column c in row k (dimension) of a staged chunk: groups of four columns, permuted
@@ -103,11 +185,11 @@ __device__ __forceinline__ int scan_row() {
 // [c0, c1).  rk, ck (rv, cv: values, [K; V] descriptor) point at row 0 and column 0 of the
 // head, D elements each.  For each tile of up to 128 columns from column t0, scan(t0, nc, w,
 // meta) is called in the threads with scan_row() >= 0: w[c] for the thread's row, meta[c] =
-// 1 / cbase[t0 + c] (if cbase is given).
+// 1 / cbase[t0 + c] (if cbase is given).  Tiles z, z + C, .. only.
 template <typename T, int D, bool KV, int RT, typename Scan>
 __device__ __forceinline__ void pair_tiles(const T* rk, const T* rv, int row0, int nrows, const T* ck, const T* cv,
                                            const float* cbase, int c0, int c1, const KParams& kp, bool vec,
-                                           float* smem, Scan scan) {
+                                           float* smem, int z, int C, Scan scan) {
   using L = Lay<D, KV, RT>;
   constexpr int TR = L::TR, TC = L::TC, CG = L::CG;
   const int tid = threadIdx.x;
@@ -132,7 +214,7 @@ __device__ __forceinline__ void pair_tiles(const T* rk, const T* rv, int row0, i
     }
   }
   const int ntiles = (c1 - c0 + CT - 1) / CT;
-  if (ntiles <= 0) return;
+  if (z >= ntiles) return;
   // column loads: 8 dimensions at a time, 8 (tid % 4) .., of columns tid / 4 + 32 u of the tile
   const int lc = tid / (KC / 8), lk = tid % (KC / 8) * 8;
   float pre[KC / 8][8];
@@ -155,9 +237,9 @@ __device__ __forceinline__ void pair_tiles(const T* rk, const T* rv, int row0, i
   const int rg = tid / CG, cg = tid % CG;
   auto row_of = [&](int i) { return (i >> 2) * (RT / 2) + 4 * rg + (i & 3); };
   const int sr = scan_row<RT>();
-  fetch(0, 0);
+  fetch(z, 0);
   int stage = 0;
-  for (int t = 0; t < ntiles; ++t) {
+  for (int t = z; t < ntiles; t += C) {
     const int t0 = c0 + t * CT;
     const int nc = min(CT, c1 - t0);
     float cm = 1.f;
@@ -175,7 +257,7 @@ __device__ __forceinline__ void pair_tiles(const T* rk, const T* rv, int row0, i
 #pragma unroll
         for (int k = 0; k < 8; ++k) cs[(lk + k) * CT + swz(u * (CT / (KC / 8)) + lc, lk + k)] = -pre[u][k];
       if (ch + 1 < L::NQ) fetch(t, ch + 1);
-      else if (t + 1 < ntiles) fetch(t + 1, 0);
+      else if (t + C < ntiles) fetch(t + C, 0);
       // one barrier per chunk: a stage is written again two chunks later
       __syncthreads();
       if (ch == L::NQ / 2) {   // the second part begins: the first waits in this thread's w slots

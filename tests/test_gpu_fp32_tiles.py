@@ -2,7 +2,7 @@
 
 Pair passes: a block takes 16, 32 or 64 rows against tiles of 128 columns, chosen by how many
 rows the call has; every choice adds a row's terms in the same order, so a head updated alone
-(16 rows a block) and among many (32 or 64) ends with the same bits.  Attention: 16, 32 or 64
+(16 rows a block, a cluster of blocks) and among many (32 or 64) ends with the same bits.  Attention: 16, 32 or 64
 queries a block, and with few blocks a cluster splits the key range; compared with float64.
 Allocation-free order: key arrays without 16-byte alignment take element loads and must give
 what aligned ones do.
@@ -51,6 +51,47 @@ def test_rows_per_block_do_not_change_a_bit(dkv, H, N, M, d, dtype, desc):
             assert torch.equal(getattr(one, name)[0, :m], getattr(many, name)[h, :m]), (h, name)
         one.close()
     many.close()
+
+
+@pytest.mark.parametrize("N,m,M,d,dtype,desc", [
+    (16, 129, 129, 64, torch.float32, 0),      # a second tile of one column
+    (1, 1025, 4000, 128, torch.bfloat16, 0),   # nine tiles over eight blocks
+    (65, 40, 3000, 128, torch.bfloat16, 0),    # blocks of the cluster without a tile
+    (300, 1152, 1300, 64, torch.float32, 1),   # whole tiles, [K; V]
+    (1000, 640, 1500, 128, torch.float32, 0),  # crossings and new baselines over clusters too
+])
+def test_clusters_hand_the_sums_on(dkv, N, m, M, d, dtype, desc):
+    """One head alone spreads its column tiles over a cluster of blocks; the same head among 200
+    fills the GPU without.  Scores, crossings and the updated bank have the same bits."""
+    g = torch.Generator(device="cuda").manual_seed(N + m)
+    k, v = (torch.randn(1, M, d, generator=g, device="cuda").to(dtype) for _ in range(2))
+    K, V = (torch.randn(1, N, d, generator=g, device="cuda").to(dtype) for _ in range(2))
+    rho = torch.rand(1, M, generator=g, device="cuda") + 1
+    got = []
+    for H in (1, 200):
+        bank = dkv.BankLayer(H, d, [M] * H, N, dtype, score_mode=dkv.DKV_SCORE_FP32, sync_heads=0, descriptor=desc)
+        bank.k.copy_(k.expand(H, -1, -1))
+        bank.v.copy_(v.expand(H, -1, -1))
+        bank.rho.copy_(rho.expand(H, -1))
+        bank.base.copy_(bank.rho / 1.2)
+        bank.import_state([m] * H)
+        bank.admit(K.expand(H, -1, -1).contiguous(), V.expand(H, -1, -1).contiguous(), 1)
+        bank.sync()
+        mid = bank.intermediates()
+        res = [mid["score"][H - 1].clone(), mid["cross"][H - 1, :m].clone()]
+        bank.compress()
+        bank.sync()
+        n = bank.occupancy_host()[H - 1]
+        got.append(res + [getattr(bank, x)[H - 1, :n].clone() for x in ("k", "rho", "base", "prov_src")])
+        bank.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    if not desc:
+        scores, perm = torch.empty(N, device="cuda"), torch.empty(N, dtype=torch.int32, device="cuda")
+        dkv.dkv_candidate_order_noalloc(k[0], (rho / 1.2)[0], m, K[0], N, d, dkv.DKV_DTYPE_FP32
+                                        if dtype == torch.float32 else dkv.DKV_DTYPE_BF16,
+                                        dkv.dkv_params_default(d), scores, perm)
+        assert torch.equal(scores, got[0][0])
 
 
 @pytest.mark.parametrize("H,Nq,occ,M,W,d,dtype", [

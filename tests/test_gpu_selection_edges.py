@@ -1,10 +1,10 @@
-"""Edges of three dispatches of the bank update.
+"""Edges of three dispatches of the bank update, and of its commit.
 
 Selection: banks of 8,192 slots and more run on a cluster of blocks per head; its lists must be
 those of Step 3 computed from the call's own crossings and projected densities, also when every
 key ties and the provenance decides.  Projection: a prefix that is the whole tested range takes
 the crossing pass's final sums, around multiples of the 128-column snapshots.  Norms: the wide
-form of the candidates' norms and the one used after an import give the same bits.
+form of the candidates' norms and the one used after an import give the same bits.  Commit: a warp copies eight rows of 128, 256 or 512 bytes.
 """
 import numpy as np
 import pytest
@@ -120,4 +120,35 @@ def test_candidate_norms_equal_the_imported_ones(dkv, N, desc):
     bank.import_state([m] * H)
     bank.sync()
     assert torch.equal(got, bank.knorm[:, :m])
+    bank.close()
+
+
+@pytest.mark.parametrize("N,M", [(1, 3), (7, 20), (9, 41), (64, 72), (130, 515)])
+@pytest.mark.parametrize("d,dtype,desc", [(64, torch.bfloat16, 0), (128, torch.bfloat16, 1), (64, torch.float32, 1),
+                                          (128, torch.float32, 0)])
+def test_every_state_is_its_candidate(dkv, N, M, d, dtype, desc):
+    """Appending and evicting commits: each state holds the key and value that its provenance
+    names, and the norm that an import computes from them."""
+    H, T = 3, 12
+    g = torch.Generator(device="cuda").manual_seed(N)
+    K, V = (torch.randn(T, H, N, d, generator=g, device="cuda").to(dtype) for _ in range(2))
+    bank = dkv.BankLayer(H, d, [M, M - 1, max(1, M // 2)], N, dtype, sync_heads=0, descriptor=desc,
+                         score_mode=dkv.DKV_SCORE_FP32 if d == 64 or dtype == torch.float32 else dkv.DKV_SCORE_TENSOR)
+    bank.reset()
+    for t in range(T):
+        bank.update(K[t], V[t], t)
+    bank.sync()
+    occ = bank.occupancy_host()
+    norms = bank.knorm.clone()
+    steps = set()
+    for h in range(H):
+        t, i = bank.prov_step[h, :occ[h]].long(), bank.prov_src[h, :occ[h]].long()
+        assert occ[h] > 0 and len(set(zip(t.tolist(), i.tolist()))) == occ[h]
+        assert torch.equal(bank.k[h, :occ[h]], K[t, h, i]) and torch.equal(bank.v[h, :occ[h]], V[t, h, i])
+        steps |= set(t.tolist())
+    assert len(steps) > 1
+    bank.import_state(occ)
+    bank.sync()
+    for h in range(H):
+        assert torch.equal(norms[h, :occ[h]], bank.knorm[h, :occ[h]])
     bank.close()

@@ -281,7 +281,13 @@ dkv_status_t dkv_bank_commit(dkv_bank_t bank, void* stream);
  *   Q  : device [H][Nq][d], Kw, Vw : device [H][W][d], O : device [H][Nq][d],
  *   all of the handle's dtype; 1 <= Nq <= 1<<20, 0 <= W <= 1<<20.
  * A head with no retained state and W = 0 gets O = 0.  Reads the current
- * committed bank; does not modify it.                                        */
+ * committed bank; does not modify it.
+ * Order of the sums: follows from the handle's H, budgets and modes, Nq, W, the
+ * device, whether the workspace has the attention scratch, and (tensor mode) the
+ * occupancies of all heads.  So the same bank and queries give the same bits
+ * however the bank came to its contents (updates, import) and also in a captured
+ * graph, but a head's low bits may differ between handles that hold it beside
+ * other heads.                                                               */
 dkv_status_t dkv_bank_attend(dkv_bank_t bank, const void* Q, int32_t Nq, const void* Kw,
                              const void* Vw, int32_t W, void* O, void* stream);
 

@@ -206,23 +206,6 @@ struct dkv_bank_s {
     if (ev_join) cudaEventDestroy(ev_join);
     if (side) cudaStreamDestroy(side);
   }
-  // Upper bounds of the occupancies as far as the calls on this handle tell (budgets at first;
-  // import, reset and commit move them), as 128-row tiles: attention's schedule estimates read
-  // them, its kernels the occupancy itself (which a replayed graph changes unseen by the host).
-  std::vector<int32_t> occ_bound;
-  int64_t bound_tiles = 0;
-  int bound_max = 0;
-  template <typename F>
-  void bound_occupancy(F f) {   // occ_bound[h] = f(h)
-    bound_tiles = 0;
-    bound_max = 0;
-    for (size_t h = 0; h < occ_bound.size(); ++h) {
-      occ_bound[h] = f(h);
-      const int tiles = (occ_bound[h] + 127) / 128;
-      bound_tiles += tiles;
-      bound_max = std::max(bound_max, tiles);
-    }
-  }
   const void* Kc = nullptr;
   const void* Vc = nullptr;
   int N = 0;
@@ -357,8 +340,6 @@ dkv_status_t dkv_bank_create(dkv_bank_t* out, int32_t H, int32_t d, const int32_
   bk->params = p;
   if (!(bk->params.sigma > 0.0f)) bk->params.sigma = std::sqrt((float)(kv ? 2 * d : d) / 2.0f);
   bk->budgets.assign(budgets, budgets + H);
-  bk->occ_bound.resize(H);
-  bk->bound_occupancy([&](size_t h) { return budgets[h]; });
   bk->tc = want_tc;
   Bank& b = bk->b;
   b.k = buf->k; b.v = buf->v; b.rho = buf->rho; b.base = buf->base; b.knorm = buf->knorm;
@@ -432,7 +413,6 @@ dkv_status_t dkv_bank_reset(dkv_bank_t bank, void* stream) {
   if (bank->state != 0) return DKV_ERR_STATE;
   cudaStream_t s = (cudaStream_t)stream;
   bank->last = s;
-  bank->bound_occupancy([](size_t) { return 0; });
   return cuda_status(cudaMemsetAsync(bank->b.occ, 0, sizeof(int32_t) * bank->b.H, s));
 }
 
@@ -507,7 +487,6 @@ static dkv_status_t commit_impl(dkv_bank_t bank, bool after, void* stream) {
   const KParams& kp = bank->kp;
   bank->last = s;
   bank->state = 0;
-  bank->bound_occupancy([&](size_t h) { return std::min(bank->budgets[h], bank->occ_bound[h] + bank->N); });
   cudaError_t e = launch_commit(b, w, bank->Vc, bank->N, bank->src_map, after, s, t);
   if (t->on && !t->attend_only) {
     // every launch timed: the two passes one after the other on `stream`, so that each
@@ -633,16 +612,9 @@ dkv_status_t dkv_bank_attend(dkv_bank_t bank, const void* Q, int32_t Nq, const v
   if (!aligned(Q, 16) || !aligned(O, 16) || (W > 0 && (!aligned(Kw, 16) || !aligned(Vw, 16)))) return DKV_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   bank->last = s;
-  cudaError_t e;
-  if (bank->tc) {
-    // a captured launch serves later steps too: its schedule follows the budgets
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const bool grows = cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
-    e = launch_attend_tc(bank->b, bank->w, grows ? bank->w.n_mtiles : bank->bound_tiles,
-                         grows ? (bank->b.M_max + 127) / 128 : bank->bound_max, Q, Nq, Kw, Vw, W, O, s, &bank->timer);
-  } else {
-    e = launch_attend_fp32(bank->b, Q, Nq, Kw, Vw, W, O, s, &bank->timer);
-  }
+  const cudaError_t e =
+      bank->tc ? launch_attend_tc(bank->b, bank->w, Q, Nq, Kw, Vw, W, O, s, &bank->timer)
+               : launch_attend_fp32(bank->b, Q, Nq, Kw, Vw, W, O, s, &bank->timer);
   return cuda_status(e);
 }
 
@@ -654,7 +626,6 @@ dkv_status_t dkv_bank_import(dkv_bank_t bank, const int32_t* occupancy, void* st
     if (occupancy[h] < 0 || occupancy[h] > bank->budgets[h]) return DKV_ERR_SHAPE;
   cudaStream_t s = (cudaStream_t)stream;
   bank->last = s;
-  bank->bound_occupancy([&](size_t h) { return occupancy[h]; });
   cudaError_t e = cudaMemcpyAsync(bank->b.occ, occupancy, sizeof(int32_t) * bank->b.H, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = launch_bank_norms(bank->b, bank->w, bank->kp, s, &bank->timer);
   if (e == cudaSuccess) e = launch_inv_base(bank->b, bank->w, s);

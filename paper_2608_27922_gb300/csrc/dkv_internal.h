@@ -144,9 +144,8 @@ cudaError_t launch_set_occupancy(const Bank& b, const int32_t* occ_dev_src, int 
 cudaError_t launch_attend_fp32(const Bank& b, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
                                void* O, cudaStream_t s, Timer* t);
 size_t attend_scratch_bytes();   // per handle: 20 MB of partial results
-// bank_tiles, bank_max: 128-row tiles of all heads' banks and of the largest, at most
-cudaError_t launch_attend_tc(const Bank& b, const Ws& w, int64_t bank_tiles, int bank_max, const void* Q, int Nq,
-                             const void* Kw, const void* Vw, int W, void* O, cudaStream_t s, Timer* t);
+cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
+                             void* O, cudaStream_t s, Timer* t);
 // Kernel launch.  after: the blocks may start before the preceding kernel of the stream has
 // ended (programmatic dependent launch), which hides the launch and the ramp behind that
 // kernel's end; every block of k must then call pdl_wait() before it reads or writes anything

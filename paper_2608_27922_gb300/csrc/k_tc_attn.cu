@@ -25,12 +25,12 @@
 // 68-cycle MMA.  Same products in the same order, measured at 2,070 MHz: 12 heads x 4,680
 // queries x 14,040 keys 283 -> 249 us (85% of 1.9 PFLOP/s), 160 heads of mixed budgets
 // 3,417 -> 3,124 us.  (The pair passes, bound by their epilogues, did not gain: unchanged.)
+#include "attn_schedule.h"
 #include "dkv_internal.h"
 #include "tc_ptx.cuh"
 
 #include <algorithm>
 #include <cmath>
-#include <climits>
 
 namespace dkv {
 
@@ -110,8 +110,9 @@ struct AttnJob {
   __nv_bfloat16* O;
   float sl2;     // log2(e) / sqrt(d)
   float* part;   // partial results of split units (nullptr: units are not split), see below
-  int4* meta;    // [CTAs] the split unit whose first part CTA i holds: {head, query tile, last
-                 //   CTA of the unit, 1}, or {.., .., .., 0}
+  int4* meta;    // [min(units, CTAs)] for each unit where there are no more than CTAs, else for the
+                 //   unit that CTA i's share ends in the middle of: {head, query tile, last CTA of
+                 //   the unit, its first CTA + 1}, or {.., .., .., 0} if the unit is not cut
 };
 
 // Equal shares of key tiles.  A unit is one 128-query tile of one head with all of that
@@ -123,24 +124,14 @@ struct AttnJob {
 // inside one CTA's share is finished there; a unit cut by a share boundary leaves fp32
 // partial results, one slot per part (part 2 i: the unit that CTA i's share begins in the
 // middle of; part 2 i + 1: the unit that it ends in the middle of), merged by tc_attend_merge.
-// A share is at least SPLIT_MIN tiles (or there is one per unit): below that a part's fixed
-// cost (query tile, first scores, partial store, about 6 us) outweighs its tiles (about 1 us
-// for two).  Units of fewer than SPLIT_UNIT tiles are not cut (a boundary inside one moves to
-// its start): they are short by themselves, and their results then do not depend on the
-// other heads of the call.
-constexpr int SPLIT_MIN = 4;
-constexpr int SPLIT_UNIT = 16;
-constexpr int SPLIT_CTAS = 152;              // most shares (the SMs of the GPU): sizes the scratch
+// Where the banks hold less than their budgets and shares do not pay (attn::shares_pay), the
+// CTAs take whole units instead, with the arithmetic of tc_attend<false> (43 heads x 35 queries,
+// mixed budgets up to 6,361 states 44% full, us: cut 35.5, whole 30.5; tc_attend<false>, which the
+// launcher would have to know the occupancies for, 26.9).
+using attn::SPLIT_CTAS;
+using attn::SPLIT_MIN;
+using attn::SPLIT_UNIT;
 constexpr int PART_FLOATS = BQ * 128 + BQ;   // O [32 column groups][128 rows] float4, then lse [128]
-
-// Estimated time of equal shares, in key tiles of one unit (0.775 us each on an SM that has
-// work, measured with 12 full heads): `per` units a CTA of nt tiles on average, one more
-// segment (each C0 tiles of fixed cost), and the store and merge of the parts.
-constexpr float C0 = 6.f, MERGE = 23.f;
-__host__ __device__ __forceinline__ float est_shares(float per, float nt) {
-  const float t = per * nt;
-  return (t > SPLIT_MIN ? t : (float)SPLIT_MIN) + (per + 1.f) * C0 + MERGE;
-}
 
 // Key tiles of a head's units.
 __device__ __forceinline__ int unit_tiles(const AttnJob& j, int h) {
@@ -178,12 +169,23 @@ struct TileCursor {
     }
   }
   // Share boundary t, 0 <= t <= total, moved to the start of its unit if that has fewer than
-  // `cut` tiles.
-  __device__ __forceinline__ int snap(const AttnJob& j, int nqt, int t, int total, int cut) {
+  // SPLIT_UNIT tiles.
+  __device__ __forceinline__ int snap(const AttnJob& j, int nqt, int t, int total) {
     if (t >= total) return total;
     const int su = seek(j, nqt, t);
-    return su < cut ? t - (t - base) % su : t;
+    return su > 0 && su < SPLIT_UNIT ? t - (t - base) % su : t;
   }
+};
+
+// Where a CTA of tc_attend<true> is in its share, kept in shared memory (only warp 0 uses it,
+// between segments; as registers it cost every warp spills), and the segment at hand: tiles
+// [first, first + nseg) of the unit of head h (-1: none left) and query tile qt, of nt in all.
+struct Walk {
+  int lo, hi;              // range tiles left of the share; or next unit, end of the units
+  int total, shares;       // tiles of the range, CTAs that have a share of it
+  int whole, by_unit;      // whole units; meta is by unit
+  int cur_h, cur_base;     // TileCursor
+  int h, qt, first, nseg, nt;
 };
 
 template <bool SPLIT>
@@ -208,7 +210,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* pv_done = bars + 13;  // [2]
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + 15);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-  volatile int* seg = reinterpret_cast<volatile int*>(tmem_holder + 2);   // [5] the segment, see below
+  volatile Walk* walk = reinterpret_cast<volatile Walk*>(tmem_holder + 2);
+  static_assert(15 * 8 + 2 * 4 + sizeof(Walk) <= 256, "barriers and walk in the space behind OFF_BAR");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int W = j.W;
@@ -226,9 +229,42 @@ __global__ void __launch_bounds__(THREADS, 1)
     fence_barrier_init();
   };
   if (warp == 1) tmem_alloc(tmem_holder, TMEM_COLS);
-  // SPLIT: this CTA's share of the range (warp 0 only)
-  int lo = 0, hi = 0, total = 0, shares = 1;
-  TileCursor cur{0, 0};
+  // SPLIT, warp 0: the next segment of this CTA's walk
+  auto next_segment = [&]() {
+    const int lo = walk->lo, hi = walk->hi;
+    TileCursor cur{walk->cur_h, walk->cur_base};
+    int sh = -1, sq = 0, sa = 0, sn = 0, su = 0, step = 0;
+    if (lo < hi && *abort_flag == 0) {
+      if (walk->whole) {
+        sh = lo / nqt;
+        sq = lo - sh * nqt;
+        sn = su = unit_tiles(j, sh);
+        step = gridDim.x;
+      } else if ((su = cur.seek(j, nqt, lo)) > 0) {
+        sh = cur.h;
+        sq = (lo - cur.base) / su;
+        sa = (lo - cur.base) - sq * su;
+        step = sn = min(su - sa, hi - lo);
+      }
+    }
+    __syncwarp();
+    if (lane != 0) return;
+    walk->lo = lo + step;
+    walk->cur_h = cur.h; walk->cur_base = cur.base;
+    walk->h = sh; walk->qt = sq; walk->first = sa; walk->nseg = sn; walk->nt = su;
+    if (sh < 0 || sa > 0) return;
+    if (sn < su) {   // a cut unit's first part: the CTAs that hold the others
+      const int total = walk->total;
+      const int last = (int)(((int64_t)(lo + su) * walk->shares + total - 1) / total) - 1;
+      j.meta[walk->by_unit ? sh * nqt + sq : blockIdx.x] = make_int4(sh, sq, last, blockIdx.x + 1);
+    } else if (walk->by_unit) {
+      j.meta[sh * nqt + sq] = make_int4(0, 0, 0, 0);
+    }
+  };
+  if (threadIdx.x == 64) {   // (warp 2: beside warp 0's look at the banks and warp 1's allocation)
+    *abort_flag = 0;
+    init_bars();
+  }
   if (SPLIT) {
     pdl_trigger();   // the merge's blocks start as SMs free up, and wait there
     if (warp == 0) {
@@ -238,26 +274,33 @@ __global__ void __launch_bounds__(THREADS, 1)
         mine += n;
         longest = max(longest, n);
       }
-      total = __reduce_add_sync(0xffffffffu, mine) * nqt;
+      const int total = __reduce_add_sync(0xffffffffu, mine) * nqt;
       longest = __reduce_max_sync(0xffffffffu, longest);
       const int units = j.b.H * nqt;
-      shares = min((int)gridDim.x, max(units, total / SPLIT_MIN));
-      // the host chose from bounds; where the banks hold less, whole units may be shorter after
-      // all (at most one per CTA: no second wave to fill)
-      const bool whole = units <= (int)gridDim.x &&
-                         (float)longest + C0 <= est_shares((float)units / gridDim.x, (float)total / units);
-      const int cut = whole ? INT_MAX : SPLIT_UNIT;
-      if ((int)blockIdx.x < shares) {
-        lo = cur.snap(j, nqt, (int)((int64_t)blockIdx.x * total / shares), total, cut);
-        TileCursor end = cur;
-        hi = end.snap(j, nqt, (int)((int64_t)(blockIdx.x + 1) * total / shares), total, cut);
+      const int shares = min((int)gridDim.x, max(units, total / SPLIT_MIN));
+      // the host chose from the budgets; where the banks hold less, whole units may be shorter
+      const bool whole =
+          !attn::shares_pay(attn::Sizes{j.b.H, nqt, (float)total / units, (float)longest}, (int)gridDim.x);
+      TileCursor cur{0, 0};
+      int lo = blockIdx.x, hi = units;
+      if (!whole) {
+        lo = hi = 0;
+        if ((int)blockIdx.x < shares) {
+          lo = cur.snap(j, nqt, (int)((int64_t)blockIdx.x * total / shares), total);
+          TileCursor end = cur;
+          hi = end.snap(j, nqt, (int)((int64_t)(blockIdx.x + 1) * total / shares), total);
+        }
       }
-      if (lane == 0) j.meta[blockIdx.x] = make_int4(0, 0, 0, 0);
+      const bool by_unit = units <= (int)gridDim.x;
+      if (lane == 0) {
+        if (!by_unit) j.meta[blockIdx.x] = make_int4(0, 0, 0, 0);
+        *abort_flag = 0;
+        walk->lo = lo; walk->hi = hi; walk->total = total; walk->shares = shares;
+        walk->whole = whole; walk->by_unit = by_unit; walk->cur_h = cur.h; walk->cur_base = cur.base;
+      }
+      __syncwarp();
+      next_segment();
     }
-  }
-  if (threadIdx.x == 0) {
-    *abort_flag = 0;
-    if (!SPLIT) init_bars();
   }
   fence_before_sync();
   __syncthreads();
@@ -265,33 +308,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t tmem = *tmem_holder;
 
   for (;;) {
-    // ---- the segment: tiles [first, first + nseg) of the unit of head h, query tile qt, which
-    // has nt_unit tiles in all; one whole unit without SPLIT
+    // ---- the segment; one whole unit without SPLIT
     int h, qt, first = 0, nseg, nt_unit;
     if (SPLIT) {
-      if (warp == 0) {
-        int sh = -1, sq = 0, sa = 0, sn = 0, su = 0;
-        if (lo < hi) {
-          su = cur.seek(j, nqt, lo);
-          sh = cur.h;
-          sq = (lo - cur.base) / su;
-          sa = (lo - cur.base) - sq * su;
-          sn = min(su - sa, hi - lo);
-          if (lane == 0 && sa == 0 && sn < su) {   // first part of a cut unit: its last CTA
-            const int64_t end = (int64_t)(lo + su) * shares;
-            j.meta[blockIdx.x] = make_int4(sh, sq, (int)((end + total - 1) / total) - 1, 1);
-          }
-          lo += sn;
-        }
-        if (lane == 0) {
-          seg[0] = sh; seg[1] = sq; seg[2] = sa; seg[3] = sn; seg[4] = su;
-          init_bars();
-        }
-      }
-      __syncthreads();
-      h = seg[0];
+      h = walk->h;
       if (h < 0) break;                          // uniform
-      qt = seg[1]; first = seg[2]; nseg = seg[3]; nt_unit = seg[4];
+      qt = walk->qt; first = walk->first; nseg = walk->nseg; nt_unit = walk->nt;
     } else {
       h = blockIdx.x / nqt;
       qt = blockIdx.x - h * nqt;
@@ -588,8 +610,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     fence_before_sync();
     __syncthreads();
     if (!SPLIT) break;
-    const bool stop = *abort_flag != 0;
-    if (threadIdx.x == 0) {
+    if (warp == 0) next_segment();               // (none after an abort)
+    if (threadIdx.x == 64) {
       mbar_inval(q_full);
       for (int g = 0; g < 2; ++g) {
         mbar_inval(k0_full + g);
@@ -599,9 +621,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         mbar_inval(p_full + g);
         mbar_inval(pv_done + g);
       }
+      init_bars();
     }
     __syncthreads();
-    if (stop) break;   // uniform
   }
   if (warp == 1) {
     fence_after_sync();
@@ -609,18 +631,21 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-// O of the units that share boundaries cut: CTA (i, y) takes rows [8 y, 8 y + 8) of the unit
-// whose first part CTA i of tc_attend holds (its last segment), the parts i, i + 1, .., last
-// added in that order with weights 2^(lse - max lse).  Thread = (row, four columns).  A row
-// whose weight is not finite in some part is 0, as a row whose sum is not is in one piece.
+// O of the units that share boundaries cut: CTA (x, y) takes rows [8 y, 8 y + 8) of the unit in
+// meta[x], the parts of tc_attend's CTAs i, i + 1, .., last added in that order with weights
+// 2^(lse - max lse).  Thread = (row, four columns).  A row whose weight is not finite in some
+// part is 0, as a row whose sum is not is in one piece.  No more blocks than the units and the
+// queries need: where no unit is cut they only start and end (43 heads x 35 queries: 1.5 us; 4 us
+// with 16 blocks per CTA of tc_attend).
 constexpr int MG_ROWS = 8;
 constexpr int MG_UNROLL = 8;
 
 __global__ void __launch_bounds__(MG_ROWS * 32) tc_attend_merge(AttnJob j) {
   pdl_wait();
-  const int i = blockIdx.x;
-  const int4 u = j.meta[i];
-  if (u.w == 0) return;
+  const int4 u = j.meta[blockIdx.x];
+  const int i = u.w - 1;                       // the CTA of the first part
+  // not cut; or never written, by a CTA that gave up (the error word tells)
+  if (i < 0 || u.z < i || u.z >= SPLIT_CTAS || u.x < 0 || u.x >= j.b.H || u.y < 0 || u.y * BQ >= j.Nq) return;
   const int n = u.z - i + 1;                   // parts
   const int row = blockIdx.y * MG_ROWS + threadIdx.x % MG_ROWS, c4 = threadIdx.x / MG_ROWS;
   const int qrow = u.y * BQ + row;
@@ -991,8 +1016,8 @@ cudaError_t tc_attn_set_smem_limits() {
 
 size_t attend_scratch_bytes() { return (size_t)SPLIT_CTAS * (2 * PART_FLOATS * sizeof(float) + sizeof(int4)); }
 
-cudaError_t launch_attend_tc(const Bank& b, const Ws& w, int64_t bank_tiles, int bank_max, const void* Q, int Nq,
-                             const void* Kw, const void* Vw, int W, void* O, cudaStream_t s, Timer* t) {
+cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
+                             void* O, cudaStream_t s, Timer* t) {
   CUtensorMap mq, mkb, mvb, mkw, mvw;
   if (!make_map_rows(&mq, Q, Nq, b.H, BQ) || !make_map_rows(&mkb, b.k, b.M_max, b.H, BK) ||
       !make_map_rows(&mvb, b.v, b.M_max, b.H, BK))
@@ -1005,51 +1030,24 @@ cudaError_t launch_attend_tc(const Bank& b, const Ws& w, int64_t bank_tiles, int
   }
   const int n_sm = sm_count();
   if (n_sm <= 0) return cudaErrorInvalidDevice;
-  const int64_t units = (int64_t)((Nq + BQ - 1) / BQ) * b.H;
-  const int64_t ctas2 = (int64_t)((Nq + 2 * BQ - 1) / (2 * BQ)) * b.H;
+  const int nqt = (Nq + BQ - 1) / BQ, wt = (W + BK - 1) / BK;
   AttnJob job{b, w.L, Nq, W, (__nv_bfloat16*)O, 1.4426950408889634f / sqrtf(128.0f), nullptr, nullptr};
-  // Schedule: the shortest of three estimates, in key tiles of one unit, from the bounds of the
-  // banks' tiles that the handle keeps.
-  //   whole units, one CTA each:   every wave lasts a unit; a lone wave its longest unit
-  //   equal shares:                all SMs busy to the end (est_shares)
-  //   two query tiles per CTA:     0.92 of the time per unit (K and V cross from L2 once for
-  //                                both), waves of two units
-  // Both sides of the lines, us (whole units | shares | two tiles), 9,360 + 4,680 keys: 12
-  // heads x 4,680 queries 249 | 264 | -; x 1,560 170 | 112 | -; x 256 95 | 37 | -; 16 heads x
-  // 4,680 - | 341 | 315; 17 heads - | 406 | 460; 7 heads x 1,846 queries x 5,903 keys 40 | 47 | -.
-  // In each, HBM: HBM_UNITS units' tiles of keys and values take it one tile's time (6.5 TB/s).
-  // Whole units in order keep the query tiles of one head side by side, which read its keys
-  // once; shares walk all heads at once, so where those do not fit L2 every unit reads its keys
-  // from HBM (whole units | shares: 123 heads x 182 queries x 15,832 keys 212 | 301, 40 x 1,560
-  // x 14,040 326 | 507; one query tile a head: 160 x 128 x 14,040 232 | 189).
-  constexpr float HBM_UNITS = 77.f;
-  constexpr double L2_BYTES = 180e6;   // (126 MB, and some reuse beyond: 24 x 1,560 x 14,040,
-                                       //  173 MB, 242 | 206)
-  const int wt = (W + BK - 1) / BK;
-  const float nt_max = (float)(bank_max + wt);
-  const float nt = (float)bank_tiles / b.H + wt;
-  const float waves = (float)((units + n_sm - 1) / n_sm), waves2 = (float)((ctas2 + n_sm - 1) / n_sm);
-  // heads read by a full wave of whole units, and by the last one
-  const float nqt = (float)((Nq + BQ - 1) / BQ), in_wave = n_sm / nqt, in_last = b.H - (waves - 1) * in_wave;
-  const float t_waves = (waves - 1) * nt * std::max(1.f, in_wave / HBM_UNITS) + nt * std::max(1.f, in_last / HBM_UNITS);
-  const float t_whole = std::max(nt_max, t_waves) + waves * C0;
-  const float t_two = ctas2 >= 2 * (int64_t)n_sm ? waves2 * (1.84f * nt + C0) : INFINITY;
-  const int n_cta = std::min(n_sm, SPLIT_CTAS);
-  const float per = (float)units / n_cta;
-  float t_share = w.attn_part && nt_max >= SPLIT_UNIT && units < 1024 ? est_shares(per, nt) : INFINITY;
-  if (2.0 * TB * b.H * nt > L2_BYTES) t_share = std::max(t_share, units * nt / HBM_UNITS + 2 * C0 + MERGE);
+  const attn::Sizes z{b.H, nqt, (float)w.n_mtiles / b.H + wt, (float)((b.M_max + BK - 1) / BK + wt)};
+  const attn::Schedule sched = attn::schedule(z, Nq, n_sm, w.attn_part != nullptr);
   timer_begin(t, "attend_tc", s);
   cudaError_t e = cudaSuccess;
-  if (t_two <= std::min(t_whole, t_share)) {
+  if (sched == attn::TWO) {
     dim3 grid((Nq + 2 * BQ - 1) / (2 * BQ), b.H);
     tc_attend2<<<grid, THREADS, SMEM2_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
-  } else if (t_whole <= t_share) {
-    tc_attend<false><<<(unsigned)units, THREADS, SMEM_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
+  } else if (sched == attn::WHOLE) {
+    tc_attend<false><<<(unsigned)nqt * b.H, THREADS, SMEM_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
   } else {
+    const int n_cta = std::min(n_sm, SPLIT_CTAS);
     job.part = w.attn_part;
     job.meta = reinterpret_cast<int4*>(w.attn_part + (size_t)SPLIT_CTAS * 2 * PART_FLOATS);
     tc_attend<true><<<n_cta, THREADS, SMEM_BYTES, s>>>(mq, mkb, mvb, mkw, mvw, job);
-    e = launch_kernel(tc_attend_merge, dim3(n_cta, BQ / MG_ROWS), MG_ROWS * 32, 0, 1, true, s, job);
+    const dim3 grid(std::min(n_cta, nqt * b.H), (std::min(Nq, BQ) + MG_ROWS - 1) / MG_ROWS);
+    e = launch_kernel(tc_attend_merge, grid, MG_ROWS * 32, 0, 1, true, s, job);
   }
   timer_end(t, s);
   return e != cudaSuccess ? e : cudaGetLastError();

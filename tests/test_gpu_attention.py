@@ -141,3 +141,52 @@ def test_shared_key_tiles_match_oracle(dkv, occ, M, Nq, W):
         ref = oracle.attend(ob.heads[h], Q[h], kw, vw)
         assert np.abs(O[h] - ref).max() < 2e-2 and np.abs(whole[h] - ref).max() < 2e-2, h
     bank.close()
+
+
+@pytest.mark.parametrize("occ", [2200, 9000])
+def test_attention_bits_follow_the_bank_alone(dkv, occ):
+    """156 units on the SMs, 9,360 states of budget: whole units pay with 2,200 states (18 key
+    tiles), equal shares with 9,000.  The same bank and queries give the same bits on the handle
+    that imported the bank, on one that was only handed its buffers, in a replayed graph, and on
+    a handle that held another bank before."""
+    H, M, d, Nq = 12, 9360, 128, 1560
+    g = torch.Generator(device="cuda")
+    g.manual_seed(occ)
+    bank = dkv.BankLayer(H, d, [M] * H, 64, torch.bfloat16)
+    bank.k.normal_(generator=g)
+    bank.v.normal_(generator=g)
+    bank.base.fill_(1.0)
+    bank.import_state([occ] * H)
+    Q = torch.randn(H, Nq, d, device="cuda", generator=g).bfloat16()
+    want = bank.attend(Q, None, None)
+    bufs = dkv.dkv_buffers_t(bank.k.data_ptr(), bank.v.data_ptr(), bank.rho.data_ptr(), bank.base.data_ptr(),
+                             bank.knorm.data_ptr(), bank.prov_step.data_ptr(), bank.prov_src.data_ptr(),
+                             bank.occupancy.data_ptr(), bank.workspace.data_ptr(), bank.workspace.numel())
+    bank.sync()
+    other = dkv.dkv_bank_create(H, d, [M] * H, 64, dkv.DKV_DTYPE_BF16, bank.params, bufs)
+    handed = torch.zeros_like(want)
+    dkv.dkv_bank_attend(other, Q, Nq, None, None, 0, handed)
+    dkv.dkv_bank_sync(other)
+    dkv.dkv_bank_destroy(other)
+    assert torch.equal(want, handed)
+
+    captured = torch.zeros_like(want)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        bank.attend(Q, None, None, captured)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(want, captured)
+
+    again = dkv.BankLayer(H, d, [M] * H, 64, torch.bfloat16)
+    again.k.copy_(bank.k)
+    again.v.copy_(bank.v)
+    again.base.fill_(1.0)
+    again.import_state([M] * H)
+    again.attend(Q, None, None)
+    again.import_state([occ] * H)
+    assert torch.equal(want, again.attend(Q, None, None))
+    bank.sync()
+    again.sync()
+    bank.close()
+    again.close()

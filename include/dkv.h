@@ -40,9 +40,11 @@
  *     dkv_bank_sync() reports; CUDA launch errors are returned as
  *     DKV_ERR_CUDA by the call that saw them.
  *   - Calls on one handle must be ordered on one stream (or by the caller's
- *     own events); attend calls among themselves too, since they share the
- *     handle's attention scratch.  admit must be followed by compress before the next admit
- *     (else DKV_ERR_STATE).  attend between admit and compress reads the
+ *     own events).  admit must be followed by compress before the next admit
+ *     (else DKV_ERR_STATE).  attend calls only read the bank and may also be on
+ *     several streams at once: those that share the handle's attention scratch
+ *     wait for each other on the device.  Replays of graphs are ordered by the
+ *     caller.  attend between admit and compress reads the
  *     pre-update bank: the update is atomic from the reader's point of view
  *     (App. C, "Decision granularity versus computational tiling").
  *   - The candidate buffers passed to admit must stay valid and unmodified

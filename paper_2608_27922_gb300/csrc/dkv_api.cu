@@ -201,7 +201,19 @@ struct dkv_bank_s {
   // disjoint slots): the latter on this library-owned stream, forked and joined by events
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // The attention scratch has one user at a time: an attend that cuts units waits, on the
+  // device, for the last one that did, whatever streams the two are on.  (A replayed graph is
+  // outside the events' reach: its replays are ordered by the caller, like all calls.)
+  struct ScratchUse {
+    cudaEvent_t done = nullptr;        // after the last such attend
+    bool used = false;
+    unsigned long long capture = 0;    // the capture it belongs to
+  };
+  std::mutex attn_mu;
+  ScratchUse attn_run, attn_cap;       // outside captures; inside
   ~dkv_bank_s() {
+    if (attn_run.done) cudaEventDestroy(attn_run.done);
+    if (attn_cap.done) cudaEventDestroy(attn_cap.done);
     if (ev_fork) cudaEventDestroy(ev_fork);
     if (ev_join) cudaEventDestroy(ev_join);
     if (side) cudaStreamDestroy(side);
@@ -360,7 +372,9 @@ dkv_status_t dkv_bank_create(dkv_bank_t* out, int32_t H, int32_t d, const int32_
   bk->kp.refresh = p.refresh_baselines;
   if (cudaStreamCreateWithFlags(&bk->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&bk->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&bk->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+      cudaEventCreateWithFlags(&bk->ev_join, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&bk->attn_run.done, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&bk->attn_cap.done, cudaEventDisableTiming) != cudaSuccess) {
     delete bk;
     return DKV_ERR_CUDA;
   }
@@ -603,6 +617,27 @@ dkv_status_t dkv_bank_update_sequential(dkv_bank_t bank, const void* Kc, const v
   return DKV_OK;
 }
 
+// Attention that cuts units, after the last one on this handle.
+static cudaError_t attend_ordered(dkv_bank_t bank, const void* Q, int Nq, const void* Kw, const void* Vw, int W, void* O,
+                                  cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(bank->attn_mu);
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  unsigned long long capture = 0;
+  cudaError_t e = cudaStreamGetCaptureInfo(s, &st, &capture);
+  const bool cap = st == cudaStreamCaptureStatusActive;
+  dkv_bank_s::ScratchUse& last = cap ? bank->attn_cap : bank->attn_run;
+  if (e == cudaSuccess && last.used && (!cap || last.capture == capture))
+    e = cudaStreamWaitEvent(s, last.done, 0);
+  if (e != cudaSuccess) return e;
+  e = launch_attend_tc(bank->b, bank->w, Q, Nq, Kw, Vw, W, O, s, &bank->timer);
+  const cudaError_t r = cudaEventRecord(last.done, s);   // (also after a launch that failed half way)
+  if (r == cudaSuccess) {
+    last.used = true;
+    last.capture = capture;
+  }
+  return e != cudaSuccess ? e : r;
+}
+
 dkv_status_t dkv_bank_attend(dkv_bank_t bank, const void* Q, int32_t Nq, const void* Kw, const void* Vw,
                              int32_t W, void* O, void* stream) {
   NvtxRange nvtx_range("dkv_bank_attend");
@@ -613,8 +648,10 @@ dkv_status_t dkv_bank_attend(dkv_bank_t bank, const void* Q, int32_t Nq, const v
   cudaStream_t s = (cudaStream_t)stream;
   bank->last = s;
   const cudaError_t e =
-      bank->tc ? launch_attend_tc(bank->b, bank->w, Q, Nq, Kw, Vw, W, O, s, &bank->timer)
-               : launch_attend_fp32(bank->b, Q, Nq, Kw, Vw, W, O, s, &bank->timer);
+      !bank->tc ? launch_attend_fp32(bank->b, Q, Nq, Kw, Vw, W, O, s, &bank->timer)
+      : attend_uses_scratch(bank->b, bank->w, Nq, W)
+          ? attend_ordered(bank, Q, Nq, Kw, Vw, W, O, s)
+          : launch_attend_tc(bank->b, bank->w, Q, Nq, Kw, Vw, W, O, s, &bank->timer);
   return cuda_status(e);
 }
 

@@ -144,6 +144,7 @@ cudaError_t launch_set_occupancy(const Bank& b, const int32_t* occ_dev_src, int 
 cudaError_t launch_attend_fp32(const Bank& b, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
                                void* O, cudaStream_t s, Timer* t);
 size_t attend_scratch_bytes();   // per handle: 20 MB of partial results
+bool attend_uses_scratch(const Bank& b, const Ws& w, int Nq, int W);   // launch_attend_tc cuts units
 cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
                              void* O, cudaStream_t s, Timer* t);
 // Kernel launch.  after: the blocks may start before the preceding kernel of the stream has

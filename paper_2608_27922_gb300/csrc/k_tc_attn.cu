@@ -1016,6 +1016,16 @@ cudaError_t tc_attn_set_smem_limits() {
 
 size_t attend_scratch_bytes() { return (size_t)SPLIT_CTAS * (2 * PART_FLOATS * sizeof(float) + sizeof(int4)); }
 
+static attn::Schedule pick_schedule(const Bank& b, const Ws& w, int Nq, int W, int n_sm) {
+  const int wt = (W + BK - 1) / BK;
+  const attn::Sizes z{b.H, (Nq + BQ - 1) / BQ, (float)w.n_mtiles / b.H + wt, (float)((b.M_max + BK - 1) / BK + wt)};
+  return attn::schedule(z, Nq, n_sm, w.attn_part != nullptr);
+}
+
+bool attend_uses_scratch(const Bank& b, const Ws& w, int Nq, int W) {
+  return pick_schedule(b, w, Nq, W, sm_count()) == attn::SHARES;
+}
+
 cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
                              void* O, cudaStream_t s, Timer* t) {
   CUtensorMap mq, mkb, mvb, mkw, mvw;
@@ -1030,10 +1040,9 @@ cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, 
   }
   const int n_sm = sm_count();
   if (n_sm <= 0) return cudaErrorInvalidDevice;
-  const int nqt = (Nq + BQ - 1) / BQ, wt = (W + BK - 1) / BK;
+  const int nqt = (Nq + BQ - 1) / BQ;
   AttnJob job{b, w.L, Nq, W, (__nv_bfloat16*)O, 1.4426950408889634f / sqrtf(128.0f), nullptr, nullptr};
-  const attn::Sizes z{b.H, nqt, (float)w.n_mtiles / b.H + wt, (float)((b.M_max + BK - 1) / BK + wt)};
-  const attn::Schedule sched = attn::schedule(z, Nq, n_sm, w.attn_part != nullptr);
+  const attn::Schedule sched = pick_schedule(b, w, Nq, W, n_sm);
   timer_begin(t, "attend_tc", s);
   cudaError_t e = cudaSuccess;
   if (sched == attn::TWO) {

@@ -190,3 +190,43 @@ def test_attention_bits_follow_the_bank_alone(dkv, occ):
     again.sync()
     bank.close()
     again.close()
+
+
+@pytest.mark.parametrize("captured", [False, True])
+def test_attention_on_two_streams_shares_the_scratch_in_turn(dkv, captured):
+    """Attends of one handle on two streams, without events between them, whose units are cut
+    (the handle's scratch holds the parts): each gives the bits that it gives alone."""
+    H, M, d, Nq, W, reps = 2, 9000, 128, 200, 300, 6
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    bank = dkv.BankLayer(H, d, [M] * H, 64, torch.bfloat16)
+    bank.k.normal_(generator=g)
+    bank.v.normal_(generator=g)
+    bank.base.fill_(1.0)
+    bank.import_state([M, M - 700])
+    Qs = [torch.randn(H, Nq, d, device="cuda", generator=g).bfloat16() for _ in range(2 * reps)]
+    Kw, Vw = (torch.randn(H, W, d, device="cuda", generator=g).bfloat16() for _ in range(2))
+    want = [bank.attend(q, Kw, Vw) for q in Qs]
+    out = [torch.zeros_like(q) for q in Qs]
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+
+    def both(main):
+        side.wait_stream(main)
+        for i in range(reps):
+            bank.attend(Qs[2 * i], Kw, Vw, out[2 * i], stream=main.cuda_stream)
+            bank.attend(Qs[2 * i + 1], Kw, Vw, out[2 * i + 1], stream=side.cuda_stream)
+        main.wait_stream(side)
+
+    if captured:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            both(torch.cuda.current_stream())
+        graph.replay()
+    else:
+        both(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    bank.sync()
+    for i, (a, b) in enumerate(zip(want, out)):
+        assert torch.equal(a, b), i
+    bank.close()

@@ -104,7 +104,7 @@ struct Timer;
 void timer_begin(Timer* t, const char* name, cudaStream_t s);
 void timer_end(Timer* t, cudaStream_t s);
 
-// ---- launches (each returns cudaGetLastError() of its launch) ----
+// ---- launches (each returns the error of its launches and leaves none pending) ----
 // update front half (admit)
 // candidates' norms and extension rows, zeroed crossing histogram, update snapshot
 // (rope != nullptr: the keys re-zeroed into w.kevict first, norms of the stored keys;
@@ -147,6 +147,13 @@ size_t attend_scratch_bytes();   // per handle: 20 MB of partial results
 bool attend_uses_scratch(const Bank& b, const Ws& w, int Nq, int W);   // launch_attend_tc cuts units
 cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
                              void* O, cudaStream_t s, Timer* t);
+// An error that the caller is told of by value: it does not stay behind as the runtime's last
+// error for a later, unrelated check to find.
+inline cudaError_t taken(cudaError_t e) {
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
+}
+
 // Kernel launch.  after: the blocks may start before the preceding kernel of the stream has
 // ended (programmatic dependent launch), which hides the launch and the ramp behind that
 // kernel's end; every block of k must then call pdl_wait() before it reads or writes anything
@@ -175,7 +182,7 @@ cudaError_t launch_kernel(void (*k)(P...), dim3 grid, unsigned threads, size_t s
   }
   cfg.attrs = at;
   cfg.numAttrs = n;
-  return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
+  return taken(cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...));
 }
 
 bool tc_supported(int d, int bf16);

@@ -1455,7 +1455,7 @@ cudaError_t launch_p(dim3 grid, cudaStream_t s, const CUtensorMap& a, const CUte
   constexpr bool after = MODE == TM_SCORE || MODE == TM_CROSS;
   if (n_units > 0) {   // persistent form (projection, survivor maintenance, new baselines)
     if constexpr (MODE == TM_PROJECT || MODE == TM_SUB || MODE == TM_NEWBASE) {
-      cudaError_t e = cudaMemsetAsync(job.w.loop_ctr + 2 * loop_slot<MODE>(), 0, 2 * sizeof(int32_t), s);
+      cudaError_t e = taken(cudaMemsetAsync(job.w.loop_ctr + 2 * loop_slot<MODE>(), 0, 2 * sizeof(int32_t), s));
       if (e != cudaSuccess) return e;
       const int64_t threads = (int64_t)n_units * BM;
       const int cblocks = (int)std::min<int64_t>((threads + 255) / 256, (int64_t)grid.x * 8);

@@ -421,6 +421,8 @@ dkv_status_t dkv_selftest_wait_timeout(int32_t limit_us, int64_t* elapsed_ns);
  * (made with that device current) looks up that array's device address and sets a
  * kernel attribute; make that first call before any stream capture.  If that set-up
  * fails the call returns DKV_ERR_CUDA and the next call on the device tries again.
+ * Device-side failure: the call has no error word.  If a bounded wait between the
+ * blocks of a score gave up, every entry of perm_out is -1 and that score is NaN.
  * Nothing in the array needs clearing: every entry a call reads is written earlier
  * in the same call.  All calls on a device share the array, so calls whose work
  * overlaps on the GPU (different streams without ordering between them) race;

@@ -30,6 +30,12 @@
 namespace dkv {
 namespace {
 
+// Score of a candidate whose sum a hand-over never reached (simt::Chain): a NaN that no
+// arithmetic returns (results are 0x7fffffff), so it is told from a NaN of the inputs.  Written
+// and recognised as integers only (nvcc 13.0 took a float compared with it bit by bit for it
+// whenever the float was any NaN).
+constexpr uint32_t NO_SCORE = 0xfffffffeu, NO_SCORE_KEY = ~NO_SCORE;   // (key: fkey's)
+
 // Scratch shared by every call on a device, held until the process exits.
 static __device__ __align__(256) float g_noalloc_scores[DKV_NOALLOC_MAX_N];
 
@@ -47,18 +53,19 @@ __global__ void __launch_bounds__(simt::NT) noalloc_score(const T* Kb, const flo
   simt::pair_tiles<T, D, false, RT>(Kc, nullptr, row0, N, Kb, nullptr, base, 0, m, kp, vec, smem, z, C,
                                     [&](int t0, int nc, const float* w, const float* inv) {
                                       const int t = t0 / simt::CT;
-                                      // (a hand-over that never came shows as NaN scores)
-                                      if (!chain.take(sr, t, acc, unused)) acc = __int_as_float(0x7fffffff);
+                                      chain.take(sr, t, acc, unused);
                                       simt::for_columns(nc, w, [&](int c, float x) { acc = __fmaf_rn(x, inv[c], acc); });
                                       chain.give(sr, t, acc, unused);
                                     });
   chain.finish();
-  if (chain.last() && sr >= 0 && row0 + sr < N) scratch[row0 + sr] = __fdiv_rn(acc, (float)m);
+  if (chain.last() && sr >= 0 && row0 + sr < N)
+    reinterpret_cast<uint32_t*>(scratch)[row0 + sr] = chain.ok ? __float_as_uint(__fdiv_rn(acc, (float)m)) : NO_SCORE;
 }
 
 // Block b places candidates [32 b, 32 b + 32): thread (i, g) = (t % 32, t / 32) counts, for
 // candidate i, those that come before it among every 8th run of ORD_RUN candidates; the
-// eight counts are added through shared memory.  2 N^2 / 32 warp comparisons in all: at
+// eight counts are added through shared memory.  Every block sees every score: if one is
+// missing (NO_SCORE) there is no order, and all of them write -1.  2 N^2 / 32 warp comparisons in all: at
 // N = 16,384 about 8 M a phase, less than the single block of a sort in shared memory took
 // for its 91 to 105 barrier-separated exchange phases.
 constexpr int ORD_RUN = 256;
@@ -80,9 +87,14 @@ __global__ void __launch_bounds__(32 * ORD_GROUPS) noalloc_order(const float* sc
   const float mine = i < N ? scratch[i] : 0.f;
   const uint32_t key = fkey(mine);
   int cnt = 0;
+  bool missing = false;
   for (int r0 = g * ORD_RUN; r0 < N; r0 += ORD_GROUPS * ORD_RUN) {   // warp-uniform
     const int n = min(ORD_RUN, N - r0);
-    for (int k = lane; k < n; k += 32) keys[g][k] = fkey(scratch[r0 + k]);
+    for (int k = lane; k < n; k += 32) {
+      const uint32_t x = fkey(scratch[r0 + k]);
+      missing = missing || x == NO_SCORE_KEY;
+      keys[g][k] = x;
+    }
     __syncwarp();
     // candidates of the run before index i precede it at equal scores
     const int below = min(max(i - r0, 0), n);
@@ -106,12 +118,14 @@ __global__ void __launch_bounds__(32 * ORD_GROUPS) noalloc_order(const float* sc
     __syncwarp();
   }
   s_cnt[g][lane] = cnt;
-  __syncthreads();
+  missing = __syncthreads_or(missing);
   if (g == 0 && i < N) {
     int pos = 0;
 #pragma unroll
     for (int q = 0; q < ORD_GROUPS; ++q) pos += s_cnt[q][lane];
-    perm[pos] = i;   // keys with their index are distinct: positions cover [0, N)
+    // (keys with their index are distinct: positions cover [0, N))
+    if (missing) perm[i] = -1;
+    else perm[pos] = i;
     if (scores) scores[i] = mine;
   }
 }

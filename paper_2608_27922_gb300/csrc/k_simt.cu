@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
       mode == PM_SCORE ? j.b.base + bh : nullptr, c0, c1, j.kp, true, smem, z, C,
       [&](int t0, int nc, const float* w, const float* meta) {
         const int t = (t0 - c0) / simt::CT;
-        if (!chain.take(sr, t, S, cross)) dev_fail(j.w.L, DEV_TIMEOUT, 6500 + mode);
+        chain.take(sr, t, S, cross);
         if (mode == PM_SCORE) {
           simt::for_columns(nc, w, [&](int c, float x) { S = __fmaf_rn(x, meta[c], S); });
         } else if (mode == PM_CROSS) {
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
           });
           static_assert(simt::CT == SNAP, "a snapshot at every tile end");
           // (a partial last tile's is the sum over all columns)
-          if (active) snap_row[(t0 + simt::CT) / SNAP] = S;
+          if (active && chain.ok) snap_row[(t0 + simt::CT) / SNAP] = S;
         } else if (mode == PM_NEWBASE) {
           simt::for_columns(nc, w, [&](int c, float x) { S = __fadd_rn(S, t0 + c == self ? 0.f : x); });
         } else {
@@ -161,6 +161,10 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
       });
   chain.finish();
   if (!active || !chain.last()) return;
+  if (!chain.ok) {   // an incomplete sum is not stored
+    dev_fail(j.w.L, DEV_TIMEOUT, 6500 + mode);
+    return;
+  }
   if ((mode == PM_SUB && (slot < 0 || slot >= hd.m_old)) || (mode == PM_NEWBASE && (self < 0 || self >= hd.M))) {
     dev_fail(j.w.L, DEV_INCONSISTENT, 6000 + mode);   // a list entry out of range: skip the write
     return;

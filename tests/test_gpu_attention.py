@@ -1,17 +1,20 @@
-"""Bank-reading attention (Sec. 3.2) on grids that take the two-query-tile kernel.
+"""Bank-reading attention (Sec. 3.2): the tensor-core schedules against the oracle.
 
-The tensor-core attention has two schedules: one CTA per 128 queries with the key
-range split between its two softmax groups (small grids), and one CTA per 256 queries
-whose two query tiles share every key tile (grids of at least two CTAs per SM).  These
-cases have enough heads to take the second one.  They use ragged bank occupancies and
-window lengths, query counts that leave a partial second tile or none, and heads with
-no keys.  Every output is compared with the oracle's softmax attention over
+There are three (csrc/attn_schedule.h): one CTA per 128 queries with the key range split
+between its two softmax groups (whole units), equal shares of the key tiles of all units with
+the cut units merged (shares; on banks that hold too little for that the same kernel takes
+whole units), and one CTA per 256 queries whose two query tiles share every key tile (two
+tiles).  Every case asserts the schedule it is there for, from the rule itself and, for the
+shares, from the list of cut units that the kernel leaves in the workspace.  The cases use
+ragged occupancies and window lengths, query counts that leave a partial second tile or none,
+and heads with no keys.  Outputs are compared with the oracle's softmax attention over
 [bank | window] in float64, within 2e-2 absolute.
 """
 import numpy as np
 import pytest
 import torch
 
+import attn_schedule as A
 import oracle
 import synth
 from gpu_util import load_state, to_dev
@@ -51,9 +54,10 @@ def _bank_with(dkv, occ, M, d=128, seed=0):
     return bank, ob
 
 
-@pytest.mark.parametrize("Nq,W", [(300, 200), (256, 0), (129, 77), (520, 128)])
-def test_two_tile_attention_matches_oracle(dkv, Nq, W):
+@pytest.mark.parametrize("Nq,W,want", [(300, 200, A.WHOLE), (256, 0, A.TWO), (129, 77, A.TWO), (520, 128, A.TWO)])
+def test_two_tile_attention_matches_oracle(dkv, Nq, W, want):
     H, M, d = 320, 400, 128   # >= 2 CTAs per SM in every case
+    assert A.launched([M] * H, Nq, W, A.n_sm()) == want
     occ = [(37 * h) % (M + 1) for h in range(H)]   # 0 .. 400, ragged
     occ[5] = 0
     bank, ob = _bank_with(dkv, occ, M, seed=Nq + W)
@@ -77,22 +81,78 @@ def test_two_tile_attention_matches_oracle(dkv, Nq, W):
     bank.close()
 
 
-def test_two_tile_attention_reads_a_long_bank(dkv):
-    """Many key tiles (bank 4,000 states + window 700) on the two-tile grid: the key and
-    value slots are reused many times over."""
-    H, M, d, Nq, W = 152, 4000, 128, 300, 700
-    occ = [M - (h % 3) * 61 for h in range(H)]
-    bank, ob = _bank_with(dkv, occ, M, seed=7)
-    rng = np.random.default_rng(8)
-    Q = _bf16(rng, (H, Nq, d), 1.5)
-    Kw, Vw = _bf16(rng, (H, W, d), 1.5), _bf16(rng, (H, W, d), 1.0)
-    O = bank.attend(to_dev(Q, torch.bfloat16), to_dev(Kw, torch.bfloat16), to_dev(Vw, torch.bfloat16))
-    O = O.float().cpu().numpy()
+def _random_bank(dkv, M, occ, seed):
+    """A bank with random states made on the GPU; heads with fewer states than M hold garbage beyond."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    bank = dkv.BankLayer(len(occ), 128, [M] * len(occ), 64, torch.bfloat16)
+    for h in range(0, len(occ), 64):
+        bank.k[h:h + 64].normal_(0, 1.5, generator=g)
+        bank.v[h:h + 64].normal_(generator=g)
+    bank.base.fill_(1.0)
+    bank.import_state(occ)
+    return bank, g
+
+
+def _rand(g, scale, *shape):
+    return (torch.randn(shape, device="cuda", generator=g) * scale).bfloat16()
+
+
+def _check(bank, occ, Q, Kw, Vw, O, heads, rows):
+    """O against the oracle at these heads and query rows."""
     bank.sync()
-    err = 0.0
-    for h in range(0, H, 7):
-        err = max(err, float(np.abs(O[h] - oracle.attend(ob.heads[h], Q[h], Kw[h], Vw[h])).max()))
-    assert err < 2e-2, err
+    assert bool(torch.isfinite(O).all())
+    for h in heads:
+        n = lambda x: x[h].double().cpu().numpy() if x is not None else np.zeros((0, 128))
+        hb = oracle.LayerBank.empty([max(1, occ[h])], 128).heads[0]
+        hb.K, hb.V = (x[h, :occ[h]].double().cpu().numpy() for x in (bank.k, bank.v))
+        got = O[h, rows].double().cpu().numpy()
+        if occ[h] == 0 and Kw is None:
+            assert np.all(got == 0), h
+            continue
+        assert np.abs(got - oracle.attend(hb, Q[h, rows].double().cpu().numpy(), n(Kw), n(Vw))).max() < 2e-2, h
+
+
+@pytest.mark.parametrize("H,M,Nq,want", [(444, 3000, 256, A.TWO), (444, 3000, 250, A.TWO), (152, 4000, 300, A.WHOLE)])
+def test_long_banks_reuse_every_slot(dkv, H, M, Nq, want):
+    """24 to 32 bank tiles and 6 of the window: the two key and three value slots of the two-tile
+    kernel (those of each group with whole units) and their parities go round many times."""
+    W = 700
+    assert A.launched([M] * H, Nq, W, A.n_sm()) == want
+    occ = [M - (h % 3) * 61 for h in range(H)]
+    bank, g = _random_bank(dkv, M, occ, 7)
+    Q, Kw, Vw = _rand(g, 1.5, H, Nq, 128), _rand(g, 1.5, H, W, 128), _rand(g, 1.0, H, W, 128)
+    with A.taken(bank) as t:
+        O = bank.attend(Q, Kw, Vw)
+    assert not t.shares
+    _check(bank, occ, Q, Kw, Vw, O, range(0, H, 21), slice(None))
+    bank.close()
+
+
+@pytest.mark.parametrize("M,occ,Nq,W,cut", [
+    (9360, [9000] * 12, 1560, 333, True),                # more units than CTAs, most CTAs hold two parts
+    (9000, [0, 9000, 0, 128, 1, 6000], 40, 0, True),     # heads without keys between cut units
+    (5000, [5000, 1500] * 4, 300, 64, True),             # units too short to cut between cut ones
+    (9000, [9000], 129, 1, True),                        # one head, a query tile of one row
+    (6000, [700] * 10, 100, 0, False),                   # budgets that pay for shares, banks that do not
+    (6000, [2100, 0, 1] * 4, 300, 5, False),
+    (9360, [2200] * 12, 1560, 0, False),                 # the same, two waves of whole units
+])
+def test_shares_of_units_match_oracle(dkv, M, occ, Nq, W, cut):
+    H = len(occ)
+    n_sm = A.n_sm()
+    assert A.launched([M] * H, Nq, W, n_sm) == A.SHARES and A.cuts(occ, Nq, W, n_sm) == cut
+    bank, g = _random_bank(dkv, M, occ, M + Nq)
+    Q = _rand(g, 1.5, H, Nq, 128)
+    Kw, Vw = (_rand(g, 1.5, H, W, 128), _rand(g, 1.0, H, W, 128)) if W else (None, None)
+    with A.taken(bank) as t:
+        O = bank.attend(Q, Kw, Vw)
+    assert t.shares and (t.cut > 0) == cut
+    rows = sorted({r for r in (0, 1, 31, 127, 128, 200, 255, 256, Nq // 2, Nq - 129, Nq - 1) if 0 <= r < Nq})
+    _check(bank, occ, Q, Kw, Vw, O, range(H), rows)
+    # a second call, on new queries, writes all of its list and parts again
+    Q = _rand(g, 1.5, H, Nq, 128)
+    _check(bank, occ, Q, Kw, Vw, bank.attend(Q, Kw, Vw), range(H), rows)
     bank.close()
 
 
@@ -100,15 +160,17 @@ def test_two_tile_attention_reads_a_long_bank(dkv):
     ([5000], 5000, 16, 700),                  # one unit, cut into many parts
     ([0], 300, 1, 0),                         # no key at all
     ([1], 300, 130, 0),                       # one key, two query tiles
-    ([0, 900, 0, 128, 1, 77], 900, 200, 0),   # heads without keys between cut units
+    ([0, 900, 0, 128, 1, 77], 900, 200, 0),   # heads without keys
     ([3000, 129], 3000, 128, 1),              # a window of one key after a bank that ends inside a tile
-    ([2000] * 13, 2000, 1560, 333),           # more query tiles than SMs: shares over unit boundaries
+    ([2000] * 13, 2000, 1560, 333),           # more query tiles than SMs
 ])
 def test_shared_key_tiles_match_oracle(dkv, occ, M, Nq, W):
-    """Grids below two CTAs per SM: the key tiles of all (head, query tile) units in equal
-    shares, units cut by share boundaries merged from fp32 parts.  The same call on a handle
-    whose workspace lacks the parts' scratch takes whole units; both match the oracle."""
+    """Few units: the first case is cut into parts, the others are whole units.  The same call on
+    a handle whose workspace lacks the parts' scratch takes whole units in every case, with the
+    same bits where the first did; both match the oracle."""
     H, d = len(occ), 128
+    cut = A.launched([M] * H, Nq, W, A.n_sm()) == A.SHARES
+    assert cut == (len(occ) == 1 and M == 5000)
     bank, ob = _bank_with(dkv, occ, M, seed=Nq + W)
     rng = np.random.default_rng(Nq)
     Q = _bf16(rng, (H, Nq, d), 1.5)
@@ -124,13 +186,16 @@ def test_shared_key_tiles_match_oracle(dkv, occ, M, Nq, W):
     bufs = dkv.dkv_buffers_t(bank.k.data_ptr(), bank.v.data_ptr(), bank.rho.data_ptr(), bank.base.data_ptr(),
                              bank.knorm.data_ptr(), bank.prov_step.data_ptr(), bank.prov_src.data_ptr(),
                              bank.occupancy.data_ptr(), spare.data_ptr(), small)
-    O = bank.attend(Qd, Kd, Vd)
+    with A.taken(bank) as t:
+        O = bank.attend(Qd, Kd, Vd)
+    assert t.shares == cut and (t.cut > 0) == cut
     whole = torch.full_like(O, 7.0)
     other = dkv.dkv_bank_create(H, d, [M] * H, 64, dkv.DKV_DTYPE_BF16, bank.params, bufs)
     dkv.dkv_bank_attend(other, Qd, Nq, Kd, Vd, W, whole)
     bank.sync()
     dkv.dkv_bank_sync(other)
     dkv.dkv_bank_destroy(other)
+    assert cut or torch.equal(O, whole)
     O, whole = O.float().cpu().numpy(), whole.float().cpu().numpy()
     for h in range(H):
         if occ[h] + W == 0:
@@ -150,6 +215,7 @@ def test_attention_bits_follow_the_bank_alone(dkv, occ):
     that imported the bank, on one that was only handed its buffers, in a replayed graph, and on
     a handle that held another bank before."""
     H, M, d, Nq = 12, 9360, 128, 1560
+    assert A.launched([M] * H, Nq, 0, A.n_sm()) == A.SHARES and A.cuts([occ] * H, Nq, 0, A.n_sm()) == (occ > 5000)
     g = torch.Generator(device="cuda")
     g.manual_seed(occ)
     bank = dkv.BankLayer(H, d, [M] * H, 64, torch.bfloat16)
@@ -197,6 +263,7 @@ def test_attention_on_two_streams_shares_the_scratch_in_turn(dkv, captured):
     """Attends of one handle on two streams, without events between them, whose units are cut
     (the handle's scratch holds the parts): each gives the bits that it gives alone."""
     H, M, d, Nq, W, reps = 2, 9000, 128, 200, 300, 6
+    assert A.launched([M] * H, Nq, W, A.n_sm()) == A.SHARES and A.cuts([M, M - 700], Nq, W, A.n_sm())
     g = torch.Generator(device="cuda")
     g.manual_seed(3)
     bank = dkv.BankLayer(H, d, [M] * H, 64, torch.bfloat16)

@@ -4,9 +4,10 @@ layers with single launches, each layer keeping its own shared prefix r* (Eq. 11
 The grouped handle is compared bit for bit with one handle per layer fed the same
 per-layer streams (those are themselves parity-tested against the oracle): bank
 contents, occupancy, provenance, densities, baselines and each layer's r* must be
-identical, and so must attention outputs whenever both handles take the same attention
-schedule (the grids of the small cases); the grouped handle is also teacher-forced
-against the oracle layer by layer.
+identical, and so must attention outputs whenever both handles take whole units of the
+same kind (the grids of the small cases: where units are cut, the cuts follow from all of
+a handle's heads); the grouped handle is also teacher-forced against the oracle layer by
+layer.
 """
 import numpy as np
 import pytest

@@ -139,7 +139,6 @@ cudaError_t launch_newbase_tc(const Bank& b, const Ws& w, const KParams& kp, cud
 // bank maintenance
 cudaError_t launch_bank_norms(const Bank& b, const Ws& w, const KParams& kp, cudaStream_t s, Timer* t);
 cudaError_t launch_inv_base(const Bank& b, const Ws& w, cudaStream_t s);
-cudaError_t launch_set_occupancy(const Bank& b, const int32_t* occ_dev_src, int value, cudaStream_t s);
 // attention
 cudaError_t launch_attend_fp32(const Bank& b, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
                                void* O, cudaStream_t s, Timer* t);

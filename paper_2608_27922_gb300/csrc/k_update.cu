@@ -29,32 +29,6 @@ constexpr int BIG = 1024;   // threads of the one-block-per-head kernels
 __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
-// Row copies as a flat loop over groups of four 16-byte chunks (64 bytes) of a row.
-// Every row is a whole number of groups and no group spans two sources, so a thread
-// resolves its row once and has four independent loads in flight before its stores.
-// map(row, group) returns the group's source and destination (src == nullptr: nothing
-// to copy) and performs the row's scalar updates for one of its groups.
-struct Group4 {
-  const uint4* src;
-  uint4* dst;
-};
-
-template <typename Map>
-__device__ __forceinline__ void copy_groups(int nrows, int per_row, Map map) {
-  const int total = nrows * per_row;
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < total; c += gridDim.x * blockDim.x) {
-    const int row = c / per_row, grp = c - row * per_row;
-    const Group4 g = map(row, grp);
-    if (g.src) {
-      uint4 v[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = g.src[k];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) g.dst[k] = v[k];
-    }
-  }
-}
-
 // One 64-byte group: all four loads are issued before the stores.
 __device__ __forceinline__ void copy64(const uint4* src, uint4* dst) {
   uint4 v[4];

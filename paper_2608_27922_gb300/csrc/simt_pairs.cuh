@@ -182,8 +182,8 @@ __device__ __forceinline__ void load8(const T* p, bool vec, float (&x)[8]) {
 // Row of the tile whose column sums this thread forms (-1: none): RT / 4 rows per warp.
 template <int RT>
 __device__ __forceinline__ int scan_row() {
-  const int lane = threadIdx.x & 31;
-  return lane < RT / 4 ? (threadIdx.x >> 5) * (RT / 4) + lane : -1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  return lane < RT / 4 ? warp * (RT / 4) + lane : -1;
 }
 
 // The interactions of rows [row0, row0 + RT) (those from nrows on are not used) with columns

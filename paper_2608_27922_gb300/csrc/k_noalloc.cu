@@ -49,17 +49,17 @@ __global__ void __launch_bounds__(simt::NT) noalloc_score(const T* Kb, const flo
   const int sr = simt::scan_row<RT>();
   simt::Chain<RT> chain(mail, z, C, (m + simt::CT - 1) / simt::CT);
   float acc = 0.f;
-  int unused = 0;
+  int lost = 0;
   simt::pair_tiles<T, D, false, RT>(Kc, nullptr, row0, N, Kb, nullptr, base, 0, m, kp, vec, smem, z, C,
                                     [&](int t0, int nc, const float* w, const float* inv) {
                                       const int t = t0 / simt::CT;
-                                      chain.take(sr, t, acc, unused);
+                                      chain.take(sr, t, acc, lost);
                                       simt::for_columns(nc, w, [&](int c, float x) { acc = __fmaf_rn(x, inv[c], acc); });
-                                      chain.give(sr, t, acc, unused);
+                                      chain.give(sr, t, acc, lost);
                                     });
   chain.finish();
   if (chain.last() && sr >= 0 && row0 + sr < N)
-    reinterpret_cast<uint32_t*>(scratch)[row0 + sr] = chain.ok ? __float_as_uint(__fdiv_rn(acc, (float)m)) : NO_SCORE;
+    reinterpret_cast<uint32_t*>(scratch)[row0 + sr] = lost != chain.LOST ? __float_as_uint(__fdiv_rn(acc, (float)m)) : NO_SCORE;
 }
 
 // Block b places candidates [32 b, 32 b + 32): thread (i, g) = (t % 32, t / 32) counts, for

@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
           });
           static_assert(simt::CT == SNAP, "a snapshot at every tile end");
           // (a partial last tile's is the sum over all columns)
-          if (active && chain.ok) snap_row[(t0 + simt::CT) / SNAP] = S;
+          if (active && cross != chain.LOST) snap_row[(t0 + simt::CT) / SNAP] = S;
         } else if (mode == PM_NEWBASE) {
           simt::for_columns(nc, w, [&](int c, float x) { S = __fadd_rn(S, t0 + c == self ? 0.f : x); });
         } else {
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(simt::NT, RT == 64 || KV ? 2 : RT == 32 ? 3 : 
       });
   chain.finish();
   if (!active || !chain.last()) return;
-  if (!chain.ok) {   // an incomplete sum is not stored
+  if (cross == chain.LOST) {   // an incomplete sum is not stored
     dev_fail(j.w.L, DEV_TIMEOUT, 6500 + mode);
     return;
   }

@@ -58,15 +58,15 @@ struct Lay {
 // adds tile t + 1 (rank (t + 1) % C of the cluster; nothing to do with C = 1).  Each scanning
 // thread sends to the same thread of that block: its two words, then the tile they are for.
 // A mailbox is free again when it is written next: that state has been through the receiver.
-// A row whose hand-over did not come within WAIT_NS (far above any legitimate wait) is not ok
-// from there on: its later hand-overs carry that (the tile negated), nobody waits again, and
-// the block that holds the row's last state must not store it.
+// A row whose hand-over did not come within WAIT_NS (far above any legitimate wait) has LOST as
+// its second word from there on (which the scans leave alone): its later hand-overs carry that,
+// nobody waits again, and the block that holds the row's last state must not store it.
 // All of a block's threads construct and finish().
 template <int RT, uint64_t WAIT_NS = 2000000000ull>
 struct Chain {
   int4* mail;      // [RT] of this block: state x, y; tile
   int z, C, tiles;
-  bool ok = true;  // this thread's row
+  static constexpr int LOST = -2147483647 - 1;
   __device__ __forceinline__ Chain(int4* m, int rank, int size, int ntiles) : mail(m), z(rank), C(size), tiles(ntiles) {
     if (C == 1) return;
     if (threadIdx.x < RT) mail[threadIdx.x].z = 0;
@@ -82,24 +82,20 @@ struct Chain {
   }
   // this block holds the state after the last tile
   __device__ __forceinline__ bool last() const { return z == (tiles > 0 ? (tiles - 1) % C : 0); }
-  // the state before tile t (unchanged if the row is not ok)
+  // the state before tile t
   __device__ __forceinline__ void take(int sr, int t, float& x, int& y) {
-    if (C == 1 || t == 0 || !ok) return;
+    if (C == 1 || t == 0 || y == LOST) return;
     const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(mail + sr));
     uint64_t t0 = 0;
     for (uint32_t it = 1;; ++it) {
       int tag;
       asm volatile("ld.acquire.cluster.shared::cta.b32 %0, [%1];" : "=r"(tag) : "r"(a + 8) : "memory");
       if (tag == t) break;
-      if (tag == -t) {
-        ok = false;
-        return;
-      }
       if ((it & 255u) == 0u) {
         const uint64_t now = globaltimer_ns();
         if (t0 == 0) t0 = now;
         if (now - t0 > WAIT_NS) {
-          ok = false;
+          y = LOST;
           return;
         }
       }
@@ -115,8 +111,7 @@ struct Chain {
         : "=r"(a)
         : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(mail + sr))), "r"((z + 1) % C));
     asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(__float_as_int(x)), "r"(y) : "memory");
-    asm volatile("st.release.cluster.shared::cluster.b32 [%0], %1;" ::"r"(a + 8), "r"(ok ? t + 1 : -(t + 1))
-                 : "memory");
+    asm volatile("st.release.cluster.shared::cluster.b32 [%0], %1;" ::"r"(a + 8), "r"(t + 1) : "memory");
   }
 };
 

@@ -37,7 +37,7 @@ __global__ void chain_probe(int tiles, int silent_tile, int silent_row, float* s
     if (sr >= 0) {
       chain.take(sr, t, x, y);
       x += (float)((sr + 1) * (t + 1));
-      y += 1;
+      if (y != chain.LOST) y += 1;
       if (t != silent_tile || sr != silent_row) chain.give(sr, t, x, y);
     }
     __syncthreads();
@@ -45,7 +45,7 @@ __global__ void chain_probe(int tiles, int silent_tile, int silent_row, float* s
   chain.finish();
   if (chain.last() && sr >= 0) {
     sums[sr] = x;
-    ok[sr] = chain.ok;
+    ok[sr] = y != chain.LOST;
     last[sr] = y;
   }
 }

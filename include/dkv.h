@@ -336,7 +336,8 @@ dkv_status_t dkv_bank_import(dkv_bank_t bank, const int32_t* occupancy, void* st
  * copy gives DKV_ERR_CUDA and leaves dst partly written.                      */
 dkv_status_t dkv_bank_export(dkv_bank_t bank, const dkv_buffers_t* dst);
 
-/* Waits for all work enqueued by this handle, then reports the sticky device
+/* Waits for the work enqueued by this handle (for the stream of its last call:
+ * order calls on other streams before that one), then reports the sticky device
  * error word (DKV_ERR_TIMEOUT / DKV_ERR_DEVICE) or a CUDA error.  Clears the
  * word after reporting it.                                                    */
 dkv_status_t dkv_bank_sync(dkv_bank_t bank);

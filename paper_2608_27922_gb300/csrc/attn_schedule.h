@@ -35,8 +35,9 @@ constexpr int SPLIT_MIN = 4;
 constexpr int SPLIT_UNIT = 16;
 constexpr int SPLIT_CTAS = 152;      // most shares (the SMs of the GPU): sizes the scratch
 constexpr int SHARE_UNITS = 1024;    // fewer units than this are cut in shares: tile numbers of the range
-                                     //   stay in an int for any bank and window (above, at 6.7 units per SM
-                                     //   and more, two tiles per CTA are estimated within 4%)
+                                     //   stay in an int for any bank and window.  Above, at 6.7 units per SM and
+                                     //   more, little is left to gain (us, two tiles per CTA | shares: 1 head x
+                                     //   262,144 queries x 9,360 keys 800 | 821, 2 x 80,000 x 18,720 978 | 961)
 constexpr float C0 = 6.f;            // fixed cost of a unit or segment
 constexpr float MERGE = 23.f;        // store and merge of the parts
 // HBM_UNITS units' tiles of keys and values take HBM one tile's time (6.5 TB/s).  Whole units

@@ -588,8 +588,8 @@ cudaError_t launch_attend_d(const Bank& b, const void* Q, int Nq, const void* Kw
     default: break;
   }
   // few queries: while there are fewer blocks than SMs, twice as many parts of the key range,
-  // each of three tiles at least (a part's merge costs about two, and shorter ranges keep one
-  // order of sums whatever the other heads of the call)
+  // each of three tiles at least (a part's merge costs about two).  Like the queries per block
+  // above, from the handle's heads and budgets and the call's sizes alone
   const int64_t blocks = (int64_t)b.H * ((Nq + 15) / 16);
   const int tiles = (int)(((int64_t)b.M_max + W + AK - 1) / AK);
   int split = 1;

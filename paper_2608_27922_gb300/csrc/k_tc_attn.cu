@@ -4,7 +4,7 @@
 //
 // One CTA owns 128 queries of one head.  The key range (bank tiles, then window
 // tiles, 128 keys each) is split in two halves, processed concurrently by two
-// softmax warpgroups that share the query tile and one MMA-issuing thread:
+// softmax warpgroups that share the query tile and one MMA-issuing warp:
 //   S_g = Q K^T            tcgen05.mma into TMEM (128 columns per group)
 //   P_g = exp2(S_g log2(e)/sqrt(d) - m_g)   softmax threads (thread = query row);
 //                          P is written back over S_g in TMEM as packed bf16
@@ -15,7 +15,7 @@
 //   O = (2^(m_0 - m) O_0 + 2^(m_1 - m) O_1) / (2^(m_0 - m) l_0 + 2^(m_1 - m) l_1).
 // Warps: 0 TMA producer, 1 MMA issuer, 2-5 softmax group 0, 6-9 softmax group 1.
 // TMEM columns: S_0 [0,128), O_0 [128,256), S_1 [256,384), O_1 [384,512).
-// The MMA-issuing thread waits once per group and tile (any wait there stalls the
+// The issuer waits once per group and tile (any wait there stalls the
 // tensor pipe): p_full_g completes when the softmax has written P_g(i) AND V(i) and
 // K(i + 1) have landed (the producer arms it with their bytes; K has two slots per
 // group, so K(i + 1) loads while S_g(i) still reads K(i)).
@@ -23,8 +23,8 @@
 // the tcgen05 instructions (elect_one).  Issued from a single divergent lane, every MMA's
 // descriptors went through that lane's registers and the issue took about 85 cycles per
 // 68-cycle MMA.  Same products in the same order, measured at 2,070 MHz: 12 heads x 4,680
-// queries x 14,040 keys 283 -> 249 us (85% of 1.9 PFLOP/s), 160 heads of mixed budgets
-// 3,417 -> 3,124 us.  (The pair passes, bound by their epilogues, did not gain: unchanged.)
+// queries x 14,040 keys 283 -> 249 us in short bursts (85% of 1.9 PFLOP/s; back to back 296 ->
+// 265, at the power limit), 160 heads of mixed budgets 3,417 -> 3,124 us.  (The pair passes, bound by their epilogues, did not gain: unchanged.)
 #include "attn_schedule.h"
 #include "dkv_internal.h"
 #include "tc_ptx.cuh"

@@ -1023,7 +1023,8 @@ static attn::Schedule pick_schedule(const Bank& b, const Ws& w, int Nq, int W, i
 }
 
 bool attend_uses_scratch(const Bank& b, const Ws& w, int Nq, int W) {
-  return pick_schedule(b, w, Nq, W, sm_count()) == attn::SHARES;
+  const int n_sm = sm_count();
+  return n_sm > 0 && pick_schedule(b, w, Nq, W, n_sm) == attn::SHARES;
 }
 
 cudaError_t launch_attend_tc(const Bank& b, const Ws& w, const void* Q, int Nq, const void* Kw, const void* Vw, int W,
